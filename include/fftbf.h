@@ -54,7 +54,10 @@ enum fftbf_status {
 };
 
 enum fftbf_precision {
-  FFTBF_PREC_FP32 = 0,    /* FP32 CUDA-core spatial FFT (default) */
+  FFTBF_PREC_FP32 = 0,    /* FP32 (default): the spatial FFT of every snapshot on the CUDA cores
+                              or, for windows of many snapshots, beams from the window's feed
+                              covariance (exact integer sums on the FP8 tensor cores, weighted
+                              and transformed once per window in two-float FP32) */
   FFTBF_PREC_TC_FP16 = 1, /* tensor-core GEMM stages, FP16 operands, FP32 accumulate */
   FFTBF_PREC_TC_BF16 = 2, /* tensor-core GEMM stages, BF16 operands, FP32 accumulate */
   FFTBF_PREC_TC_FP16X3 = 3 /* tensor-core GEMM stages on split FP16 operands (hi + lo,

@@ -6,6 +6,7 @@
 
 #include "beam_fp32.cuh"
 #include "beam_fp32_warp.cuh"
+#include "corr.cuh"
 
 namespace fftbf {
 
@@ -86,6 +87,8 @@ extern template int launch_fft_mx<16>(const BeamArgs&, int, int, cudaStream_t);
 
 int launch_beams_fp32(const BeamArgs& a, int nsm, cudaStream_t st) {
   if (a.nwin <= 0) return FFTBF_OK;
+  if (a.err && !getenv_flag("FFTBF_FP32_GENERIC") && corr_preferred(a))
+    return launch_beams_corr(a, a.err, nsm, st);
   if (fp32_n512_supported(a) && !getenv_flag("FFTBF_FP32_GENERIC"))
     return launch_beams_fp32_n512(a, nsm, st);
   if (fp32_warp_supported(a) && !getenv_flag("FFTBF_FP32_GENERIC"))
@@ -158,6 +161,22 @@ __global__ void tables_kernel(int nx, int mx, int my, float2* ex, float2* tw) {
 int build_tables(int nx, int mx, int my, float2* ex, float2* tw, cudaStream_t st) {
   const int n = my > mx * nx ? my : mx * nx;
   tables_kernel<<<(n + 255) / 256, 256, 0, st>>>(nx, mx, my, ex, tw);
+  FFTBF_CUDA_TRY(cudaGetLastError());
+  return FFTBF_OK;
+}
+
+// Two-float tables of the covariance form: value = hi + lo, both from FP64.
+__global__ void corr_table_kernel(int mx, int my, float4* cw) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= my + mx) return;
+  double s, c;
+  sincospi(i < my ? 2.0 * (double)i / (double)my : 2.0 * (double)(i - my) / (double)mx, &s, &c);
+  const float ch = (float)c, sh = (float)-s;
+  cw[i] = make_float4(ch, (float)(c - (double)ch), sh, (float)(-s - (double)sh));
+}
+
+int build_corr_table(int mx, int my, float4* cw, cudaStream_t st) {
+  corr_table_kernel<<<(mx + my + 255) / 256, 256, 0, st>>>(mx, my, cw);
   FFTBF_CUDA_TRY(cudaGetLastError());
   return FFTBF_OK;
 }

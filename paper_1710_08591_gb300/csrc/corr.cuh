@@ -1,0 +1,43 @@
+// Interface of the covariance form of the FP32 path (beam_corr.cu).
+#pragma once
+
+#include <cuda.h>
+
+#include "internal.cuh"
+
+namespace fftbf {
+
+// One array of a launch and how its lattice is cut (filled by corr_make_job).
+struct CorrJob {
+  CUtensorMap map;      // the voltages (tma)
+  BeamArgs a;
+  int ny, nyp;          // N-S feeds, and their slots (a multiple of 16, 32 or 64)
+  int nant, np, nt;     // feeds, slots, tiles of 256 slots per axis
+  int nch;              // chunks of 32 snapshots per window
+  int mode;             // epilogue split 0..2: 8-slot groups per run 4x8, 4x4, 2x2
+  int tma;              // voltages staged by TMA
+  int64_t item0, nitems;
+};
+struct CorrSizes {      // shared-memory sizes, the largest over the launch's jobs
+  int ns, nr;           // operand stages, staged voltage tiles
+  int wslots, vlen, stg, slice;
+  int cplx;             // some weights are complex
+  int tma;              // every job's voltages are staged by TMA
+};
+struct CorrParams {
+  CorrJob one;          // the only job, or
+  const CorrJob* table; // a device table of njobs
+  int njobs;
+  int64_t total;        // work items
+  int* err;
+  CorrSizes s;
+};
+
+bool corr_make_job(const BeamArgs& a, CorrJob* J);
+bool corr_sizes(const CorrJob* jobs, int n, CorrSizes* out);
+int corr_maps(CorrJob* jobs, int n, const CorrSizes& s);
+int corr_launch(CorrParams& p, int nsm, cudaStream_t st);
+bool corr_preferred(const BeamArgs& a);
+int launch_beams_corr(const BeamArgs& a, int* err, int nsm, cudaStream_t st);
+
+}  // namespace fftbf

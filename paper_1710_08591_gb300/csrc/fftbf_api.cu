@@ -97,6 +97,7 @@ fftbf_plan* fftbf_plan_create(int nx, int ny, int pad_x, int pad_y, int npol, in
   if (e == cudaSuccess) e = cudaMalloc(&p->d_w, sizeof(float2) * nant);
   if (e == cudaSuccess) e = cudaMalloc(&p->d_ex, sizeof(float2) * pad_x * nx);
   if (e == cudaSuccess) e = cudaMalloc(&p->d_tw, sizeof(float2) * pad_y);
+  if (e == cudaSuccess) e = cudaMalloc(&p->d_cw, sizeof(float4) * (pad_y + pad_x));
   if (e == cudaSuccess) e = cudaMalloc(&p->d_err, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(p->d_err, 0, sizeof(int));
   if (e == cudaSuccess) {
@@ -115,6 +116,7 @@ fftbf_plan* fftbf_plan_create(int nx, int ny, int pad_x, int pad_y, int npol, in
     return nullptr;
   }
   if (build_tables(nx, pad_x, pad_y, p->d_ex, p->d_tw, 0) != FFTBF_OK ||
+      build_corr_table(pad_x, pad_y, p->d_cw, 0) != FFTBF_OK ||
       (e = cudaDeviceSynchronize()) != cudaSuccess) {
     if (e != cudaSuccess) cuda_error(e, "plan tables");
     fftbf_destroy(p);
@@ -202,6 +204,8 @@ int fftbf_execute(fftbf_plan* p, const uint8_t* volts, int64_t T, float* beams, 
   a.nwin = T / p->n_int;
   a.ew_dft = (p->mx == p->nx) && (p->mx & (p->mx - 1)) == 0 && p->mx <= 16;
   a.real_w = p->real_w ? 1 : 0;
+  a.cw = p->d_cw;
+  a.err = p->d_err;
   const int nsnap = p->n_int * p->npol;
   int S = kMaxElems / (p->mx * p->my);
   if (S < 1) S = 1;
@@ -317,6 +321,7 @@ void fftbf_destroy(fftbf_plan* p) {
     cudaFree(p->d_w);
     cudaFree(p->d_ex);
     cudaFree(p->d_tw);
+    cudaFree(p->d_cw);
     cudaFree(p->d_b1);
     cudaFree(p->d_b2);
     cudaFree(p->d_b1lo);

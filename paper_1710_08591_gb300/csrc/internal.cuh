@@ -55,6 +55,8 @@ struct BeamArgs {
   int ew_dft;             // 1 if mx == nx and mx is a power of two (E-W is a plain DFT)
   int real_w;             // 1 if every weight is real (two multiplies instead of a complex one)
   int64_t nwin;           // windows in this call
+  const float4* cw;       // two-float exp(-2 pi i k / my), k < my, then exp(-2 pi i k / mx): (cos hi, lo, -sin hi, lo)
+  int* err;               // device error word of bounded waits; null: no kernel that needs one
 };
 
 // Launch the FP32 fused beam kernel. Returns FFTBF_OK or an error code.
@@ -116,6 +118,7 @@ int launch_debug_tc_gemm(const uint16_t* A, const uint16_t* B, int n, bool bf16,
 int launch_debug_wait_timeout(uint64_t limit_ns, int* err, cudaStream_t st);
 // FP64 table builders (device), rounded to FP32.
 int build_tables(int nx, int mx, int my, float2* ex, float2* tw, cudaStream_t st);
+int build_corr_table(int mx, int my, float4* cw, cudaStream_t st);
 
 // Tied-beam weight tables and regridding GEMM.
 struct AxisWindow {
@@ -201,6 +204,7 @@ struct fftbf_plan {
   float2* d_w = nullptr;
   float2* d_ex = nullptr;
   float2* d_tw = nullptr;
+  float4* d_cw = nullptr;         // two-float twiddles of the covariance form (my, then mx)
   fftbf::TiedTables tied;
   fftbf::HostPipe pipe;
   std::vector<float> h_w;         // host copy of the weights (re, im interleaved)

@@ -1,0 +1,108 @@
+"""The covariance form of the FP32 path (beam_corr.cu), forced at the sizes where its tiles,
+runs and stages can go wrong, against the oracle and the FFT kernels."""
+import numpy as np
+import pytest
+
+import synth
+from helpers import TOL_BEAM, make_case, oracle_beams, rel_err_per_beam
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import paper_1710_08591_gb300 as fb  # noqa: E402
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    fb.build()
+    fb.lib()
+
+
+def run(v, w, nx, ny, mx, my, npol, nfreq, n_int, offset=0):
+    T = v.shape[0]
+    flat = torch.from_numpy(np.ascontiguousarray(v).reshape(-1))
+    base = torch.zeros(flat.numel() + 16, dtype=torch.uint8, device="cuda")
+    dv = base[offset:offset + flat.numel()]
+    dv.copy_(flat)
+    out = torch.full((T // n_int, nfreq, mx, my), float("nan"), device="cuda")
+    with fb.plan_create(nx, ny, mx, my, npol, nfreq, n_int, weights=w) as plan:
+        fb.execute(plan, dv, T, out)
+        fb.plan_sync(plan)
+    return out.cpu().numpy()
+
+
+CASES = [
+    # nx, ny, mx, my, npol, nfreq, n_int, windows, weights
+    (1, 16, 1, 32, 1, 1, 31, 1, "uniform"),      # one tile, 32 columns, part of one K step
+    (2, 16, 2, 32, 1, 200, 33, 2, "random"),     # several items per CTA pair, second K step begun
+    (16, 16, 16, 32, 2, 2, 48, 1, "half_sine"),  # 16-slot rows, one full tile
+    (17, 16, 17, 32, 1, 2, 64, 1, "random"),     # 272 slots: a second tile column of 32
+    (4, 32, 4, 64, 2, 2, 40, 1, "half_sine"),    # 32-slot rows
+    (9, 32, 9, 63, 1, 2, 65, 1, "random"),       # 288 slots, odd beam counts
+    (8, 64, 8, 128, 2, 2, 50, 2, "half_sine"),   # 64-slot rows
+    (5, 64, 4, 128, 1, 2, 70, 1, "random"),      # 320 slots, E-W folded
+    (3, 128, 3, 256, 2, 2, 36, 1, "half_sine"),  # 128-slot rows, a half-wide tile column
+    (3, 128, 4, 256, 4, 1, 20, 1, "random"),     # four polarisations, E-W padded
+    (4, 256, 4, 512, 2, 2, 96, 2, "half_sine"),  # 256-slot rows: one pair of rows per tile
+    (2, 512, 2, 1024, 1, 1, 40, 1, "half_sine"), # rows longer than a tile
+    (1, 1024, 1, 2048, 1, 1, 33, 1, "random"),
+    (4, 80, 7, 159, 1, 2, 45, 1, "half_sine"),   # rows of 80: runs of 16, 320 slots
+    (3, 96, 3, 192, 2, 2, 40, 1, "half_sine"),   # rows of 96: runs of 32
+    (3, 37, 5, 73, 1, 3, 100, 2, "random"),      # not a multiple of 16: direct loads, minimum padding
+    (2, 100, 2, 256, 3, 2, 25, 1, "half_sine"),  # direct loads, three polarisations, rows padded to 128
+    (2, 200, 2, 512, 1, 2, 64, 1, "random"),     # rows padded to 256
+    (6, 20, 4, 8, 1, 2, 96, 1, "random"),        # cyclic co-adding on both axes
+    (1, 1, 1, 1, 1, 2, 64, 1, "random"),         # one feed, one beam
+]
+
+
+@pytest.mark.parametrize("case", CASES, ids=lambda c: "x".join(map(str, c[:4])) + f"_p{c[4]}_n{c[6]}_{c[8]}")
+def test_covariance_matches_oracle(case, monkeypatch):
+    """TOL_BEAM is the FP32 bound of every beam; the sums here are exact integers, weighted in
+    FP32 and summed and transformed in two-float arithmetic, so what is left is the rounding
+    of the weighted products (about 2^-24 each, random)."""
+    monkeypatch.setenv("FFTBF_FP32_PATH", "cov")
+    nx, ny, mx, my, npol, nfreq, n_int, nwin, wk = case
+    v, w = make_case(nx, ny, mx, my, npol, nfreq, n_int * nwin, n_int, weights=wk, seed=17)
+    got = run(v, w, nx, ny, mx, my, npol, nfreq, n_int)
+    ref = oracle_beams(v, w, nx, ny, mx, my, npol, nfreq, n_int)
+    assert np.all(np.isfinite(got))
+    err = rel_err_per_beam(got, ref)
+    assert err.max() <= TOL_BEAM, f"max rel err {err.max():.3g}"
+
+
+def test_misaligned_voltages_give_identical_beams(monkeypatch):
+    """Off a 16-byte boundary the voltages are loaded directly instead of by TMA."""
+    monkeypatch.setenv("FFTBF_FP32_PATH", "cov")
+    shape = (4, 64, 4, 128, 2, 3, 40)
+    nx, ny, mx, my, npol, nfreq, n_int = shape
+    v, w = make_case(nx, ny, mx, my, npol, nfreq, 2 * n_int, n_int, weights="random", seed=5)
+    assert np.array_equal(run(v, w, *shape), run(v, w, *shape, offset=3))
+
+
+def test_saturated_source_no_worse_than_the_transform(monkeypatch):
+    """A full-scale coherent source over quantised noise: the covariance's weak beams are
+    small differences of large sums. Its error against the oracle stays within the FFT
+    kernels' bound of 1e-5 of every beam."""
+    shape = (4, 256, 4, 512, 2, 1, 192)
+    nx, ny, mx, my, npol, nfreq, n_int = shape
+    v = synth.volts(n_int, nfreq, npol, nx, ny, seed=8, sigma=1.0, sources=[(0.137, 0.291, 5.0)])
+    w = synth.separable_weights(synth.half_sine(nx), synth.half_sine(ny))
+    ref = oracle_beams(v, w, nx, ny, mx, my, npol, nfreq, n_int)
+    monkeypatch.setenv("FFTBF_FP32_PATH", "cov")
+    assert rel_err_per_beam(run(v, w, *shape), ref).max() <= TOL_BEAM
+
+
+def test_constant_input_is_exact(monkeypatch):
+    """Every voltage at -8 - 8i, the largest product: uniform weights put all power in beam
+    (0, 0) and exactly none elsewhere; nothing is negative."""
+    monkeypatch.setenv("FFTBF_FP32_PATH", "cov")
+    nx, ny, n_int = 4, 16, 300
+    v = np.full((n_int, 1, 1, nx, ny), 0x88, np.uint8)
+    got = run(v, None, nx, ny, nx, ny, 1, 1, n_int)[0, 0]
+    assert got[0, 0] == n_int * 128 * (nx * ny) ** 2
+    rest = got.copy()
+    rest[0, 0] = 0
+    assert rest.min() >= 0 and rest.max() <= 1e-12 * got[0, 0]
