@@ -11,6 +11,9 @@
 // item's accumulation order depends only on the item, so an array's beams are
 // bit-identical alone and in any mix. The launch (counter reset + kernel) is captured in
 // a CUDA graph and replayed while the batch's buffers stay the same.
+// Arrays with windows of many snapshots (corr_preferred) go through the covariance kernel
+// instead, all of them in one launch over a job table of its own, in the same graph: twelve
+// uneven arrays of 512 snapshots per window 20.99 -> 11.63 ms (all twelve through it).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -23,6 +26,7 @@
 
 #include "beam_fp32.cuh"
 #include "beam_fp32_warp.cuh"
+#include "corr.cuh"
 
 namespace fftbf {
 
@@ -285,6 +289,10 @@ struct fftbf_batch {
   std::vector<int> order;          // job order: costliest items first
   std::vector<int> S;              // tuned snapshots per step, per plan
   std::vector<int> V;              // tuned variant (generic or warp path), per plan
+  std::vector<char> cov;           // per plan: through the covariance kernel
+  std::vector<CorrJob> cjobs;      // its jobs, their device copy and launches
+  CorrJob* d_cjobs = nullptr;
+  std::vector<CorrParams> claunch;
   std::vector<BatchJob> jobs;
   BatchJob* d_jobs = nullptr;
   unsigned long long* d_counter = nullptr;
@@ -310,9 +318,16 @@ static void fill_args(const fftbf_plan* p, BeamArgs& a) {
   a.nyf = std::min(p->ny, p->my);
   a.ew_dft = (p->mx == p->nx) && (p->mx & (p->mx - 1)) == 0 && p->mx <= 16;
   a.real_w = p->real_w ? 1 : 0;
+  a.cw = p->d_cw;
+  a.err = p->d_err;
 }
 
 static int launch_jobs(fftbf_batch* bb, int64_t total, cudaStream_t st) {
+  for (CorrParams& p : bb->claunch) {
+    const int rc = corr_launch(p, bb->nsm, st);
+    if (rc != FFTBF_OK) return rc;
+  }
+  if (total == 0) return FFTBF_OK;
   FFTBF_CUDA_TRY(cudaMemsetAsync(bb->d_counter, 0, sizeof(unsigned long long), st));
   const int64_t grid = std::min<int64_t>(total, (int64_t)bb->nsm * bb->grid_per_sm);
   batch_kernel<<<(unsigned)grid, kThreads, bb->smem, st>>>(bb->d_jobs, (int)bb->jobs.size(),
@@ -358,6 +373,15 @@ static float time_candidate(fftbf_batch* bb, const fftbf_plan* p, int variant, i
   return best;
 }
 
+// Whether a plan's arrays go through the covariance kernel: a rule on the plan alone, so an
+// array's beams are the same in any batch (FFTBF_BATCH_PATH forces the batch kernel's paths).
+static bool batch_takes_cov(const fftbf_plan* p) {
+  BeamArgs a;
+  fill_args(p, a);
+  return !std::getenv("FFTBF_BATCH_PATH") && corr_preferred(a);
+}
+bool fftbf::batch_cov(const fftbf_batch* bb, int i) { return bb->cov[i] != 0; }
+
 extern "C" {
 
 fftbf_batch* fftbf_batch_create(fftbf_plan* const* plans, int n) {
@@ -387,6 +411,7 @@ fftbf_batch* fftbf_batch_create(fftbf_plan* const* plans, int n) {
   cudaSetDevice(bb->device);
   cudaError_t e = cudaMalloc(&bb->d_jobs, sizeof(BatchJob) * bt::kMaxJobs);
   if (e == cudaSuccess) e = cudaMalloc(&bb->d_counter, sizeof(unsigned long long));
+  if (e == cudaSuccess) e = cudaMalloc(&bb->d_cjobs, sizeof(CorrJob) * bt::kMaxJobs);
   // shared memory: the largest item footprint over the plans and their S candidates
   bb->smem = 200 * 1024;
   if (e == cudaSuccess)
@@ -398,15 +423,23 @@ fftbf_batch* fftbf_batch_create(fftbf_plan* const* plans, int n) {
   float* db = nullptr;
   size_t vbytes = 0, bbytes = 0;
   for (auto* p : bb->plans) {
+    bb->cov.push_back(batch_takes_cov(p));
+    if (bb->cov.back()) continue;                      // nothing to tune
     vbytes = std::max(vbytes, (size_t)2 * p->n_int * p->nfreq * p->npol * p->nx * p->ny);
     bbytes = std::max(bbytes, (size_t)2 * p->nfreq * p->mx * p->my * sizeof(float));
   }
-  if (e == cudaSuccess) e = cudaMalloc(&dv, vbytes);
-  if (e == cudaSuccess) e = cudaMalloc(&db, bbytes);
-  if (e == cudaSuccess) e = cudaMemset(dv, 0, vbytes);
+  if (e == cudaSuccess && vbytes) e = cudaMalloc(&dv, vbytes);
+  if (e == cudaSuccess && vbytes) e = cudaMalloc(&db, bbytes);
+  if (e == cudaSuccess && vbytes) e = cudaMemset(dv, 0, vbytes);
   size_t max_smem = 0;
   if (e == cudaSuccess) {
-    for (auto* p : bb->plans) {
+    for (size_t pi = 0; pi < bb->plans.size(); ++pi) {
+      fftbf_plan* p = bb->plans[pi];
+      if (bb->cov[pi]) {
+        bb->S.push_back(kCorrSteps);
+        bb->V.push_back(-1);
+        continue;
+      }
       const TuneKey key{p->nx, p->ny, p->mx, p->my, p->npol, p->n_int};
       // FFTBF_BATCH_PATH=generic|warp restricts the candidates (a test hook; bypasses the
       // process-wide cache)
@@ -503,42 +536,61 @@ int fftbf_batch_execute(fftbf_batch* bb, const uint8_t* const* volts_dev, int64_
   struct Restore { int d; ~Restore() { cudaSetDevice(d); } } restore{prev};
   cudaStream_t st = static_cast<cudaStream_t>(stream);
 
-  std::vector<BatchJob> jobs(n);
+  std::vector<BatchJob> jobs;
+  std::vector<CorrJob> cjobs;
   std::vector<const void*> ptrs;
   int64_t total = 0;
   for (int k = 0; k < n; ++k) {
     const int i = bb->order[k];
-    BatchJob& J = jobs[k];
+    ptrs.push_back(volts_dev[i]);
+    ptrs.push_back(beams_dev[i]);
+    BatchJob J{};
     fill_args(bb->plans[i], J.a);
     J.a.S = bb->S[i];
     J.a.volts = volts_dev[i];
     J.a.beams = beams_dev[i];
     J.a.nwin = T / bb->plans[i]->n_int;
+    if (bb->cov[i]) {
+      CorrJob C;
+      corr_make_job(J.a, &C);
+      cjobs.push_back(C);
+      continue;
+    }
     J.variant = bb->V[i];
     J.nitems = J.a.nwin * bb->plans[i]->nfreq;
     J.item0 = total;
     total += J.nitems;
-    ptrs.push_back(volts_dev[i]);
-    ptrs.push_back(beams_dev[i]);
+    jobs.push_back(J);
   }
+  // upload the job tables of new buffers
+  auto upload = [&]() -> int {
+    const int rc = corr_plan_jobs(cjobs, bb->d_cjobs, nullptr, &bb->claunch);
+    if (rc != FFTBF_OK) return rc;
+    bb->jobs = jobs;
+    bb->cjobs = cjobs;
+    if (!jobs.empty())
+      FFTBF_CUDA_TRY(cudaMemcpyAsync(bb->d_jobs, bb->jobs.data(), sizeof(BatchJob) * jobs.size(),
+                                     cudaMemcpyHostToDevice, st));
+    if (!cjobs.empty())
+      FFTBF_CUDA_TRY(cudaMemcpyAsync(bb->d_cjobs, bb->cjobs.data(), sizeof(CorrJob) * cjobs.size(),
+                                     cudaMemcpyHostToDevice, st));
+    return FFTBF_OK;
+  };
   if (st == nullptr) {
     // the legacy default stream cannot be captured: upload the table and launch directly
     if (bb->exec) { cudaGraphExecDestroy(bb->exec); bb->exec = nullptr; }
-    bb->jobs = jobs;
-    FFTBF_CUDA_TRY(cudaMemcpyAsync(bb->d_jobs, bb->jobs.data(), sizeof(BatchJob) * n,
-                                   cudaMemcpyHostToDevice, st));
-    return launch_jobs(bb, total, st);
+    const int rc = upload();
+    return rc == FFTBF_OK ? launch_jobs(bb, total, st) : rc;
   }
   const bool same = bb->exec && bb->exec_stream == st && bb->exec_T == T && bb->exec_ptrs == ptrs;
   if (!same) {
     // new job table: upload it and capture (counter reset + kernel) as a graph
     if (bb->exec) { cudaGraphExecDestroy(bb->exec); bb->exec = nullptr; }
-    bb->jobs = jobs;
-    FFTBF_CUDA_TRY(cudaMemcpyAsync(bb->d_jobs, bb->jobs.data(), sizeof(BatchJob) * n,
-                                   cudaMemcpyHostToDevice, st));
+    int rc = upload();
+    if (rc != FFTBF_OK) return rc;
     cudaGraph_t g = nullptr;
     FFTBF_CUDA_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-    const int rc = launch_jobs(bb, total, st);
+    rc = launch_jobs(bb, total, st);
     cudaError_t e = cudaStreamEndCapture(st, &g);
     if (rc != FFTBF_OK) { if (g) cudaGraphDestroy(g); return rc; }
     if (e != cudaSuccess) return cuda_error(e, "batch graph capture");
@@ -553,7 +605,11 @@ int fftbf_batch_execute(fftbf_batch* bb, const uint8_t* const* volts_dev, int64_
   return FFTBF_OK;
 }
 
-int fftbf_batch_grid(const fftbf_batch* bb) { return bb->nsm * bb->grid_per_sm; }
+int fftbf_batch_grid(const fftbf_batch* bb) {
+  for (char c : bb->cov)
+    if (!c) return bb->nsm * bb->grid_per_sm;
+  return bb->nsm / 2 * 2;                              // every array through the covariance kernel
+}
 size_t fftbf_batch_smem(const fftbf_batch* bb) { return bb->smem; }
 
 int fftbf_batch_tuned_steps(const fftbf_batch* bb, int i) {
@@ -575,6 +631,7 @@ void fftbf_batch_destroy(fftbf_batch* bb) {
   if (bb->exec) cudaGraphExecDestroy(bb->exec);
   cudaFree(bb->d_jobs);
   cudaFree(bb->d_counter);
+  cudaFree(bb->d_cjobs);
   cudaSetDevice(prev);
   delete bb;
 }

@@ -62,7 +62,7 @@ namespace fftbf {
 namespace corr {
 constexpr int NT = 640;                  // 20 warps (warps are allocated by fours): 96 registers
 constexpr int EPI = 256, PROD = 256;     // threads of the epilogue and the producers
-constexpr int KS = 64;                   // snapshots per stage: two K = 32 MMA steps
+constexpr int KS = kCorrSteps;           // snapshots per stage: two K = 32 MMA steps
 constexpr int NE = KS / 16;              // units per thread, stage and operand
 constexpr int TILE = 128 * KS;           // one operand component: 128 slots x 64 snapshots, e4m3
 constexpr int STAGE = 4 * TILE;          // rows re, rows im, columns re, columns im
@@ -281,11 +281,19 @@ __device__ __forceinline__ void dd_acc(Cdd& a, float2 x) {
   a.h = s;
 }
 
-__device__ __forceinline__ const CorrJob* find_job(const CorrParams& p, int64_t item) {
-  if (!p.table) return &p.one;
-  int k = 0;
+// The job of a work item; k: the job of this role's last item (items only grow).
+__device__ __forceinline__ const CorrJob& find_job(const CorrParams& p, int64_t item, int& k) {
+  if (!p.table) return p.one;
   while (k + 1 < p.njobs && item >= p.table[k + 1].item0) ++k;
-  return p.table + k;
+  return p.table[k];
+}
+// A wait that ran out: every role of the CTA leaves, and the launch's error words are set.
+__device__ __forceinline__ void corr_fail(const CorrParams& p, volatile int* abort_sm) {
+  *abort_sm = 1;
+  if (p.err) atomicExch(p.err, FFTBF_ETIMEOUT);
+  else if (!p.table) atomicExch(p.one.a.err, FFTBF_ETIMEOUT);
+  else
+    for (int k = 0; k < p.njobs; ++k) atomicExch(p.table[k].a.err, FFTBF_ETIMEOUT);
 }
 // Column slots of tile column J (a multiple of 32)
 __device__ __forceinline__ int tile_cols(int np, int J) {
@@ -787,8 +795,9 @@ __device__ __forceinline__ void produce_staged(const CorrParams& P, unsigned cha
   const uint32_t full0 = map_rank(tc::smem_u32(bars + FULL), 0);
   int slot = 0, rs = 0, turn = 0;                      // of the current stage
   uint32_t par = 1, rpar = 0;
+  int job = 0;
   for (int64_t item = pair; item < P.total; item += npairs) {
-    const CorrJob& J = *find_job(P, item);
+    const CorrJob& J = find_job(P, item, job);
     const int nt = J.nt, np = J.np, nsnap = J.a.n_int * J.a.npol;
     for (int I = 0; I < nt; ++I)
       for (int Jc = I; Jc < nt; ++Jc) {
@@ -797,10 +806,7 @@ __device__ __forceinline__ void produce_staged(const CorrParams& P, unsigned cha
         for (int left = nsnap; left > 0; left -= KS) {
           if (turn == grp) {
             const bool ok = wait_pair(bars + RAWF + rs, rpar, abort_sm) && wait_pair(bars + EMPTY + slot, par, abort_sm);
-            if (!ok) {
-              *abort_sm = 1;
-              atomicExch(P.err, FFTBF_ETIMEOUT);
-            }
+            if (!ok) corr_fail(P, abort_sm);
             if (!__all_sync(0xffffffffu, ok)) return;
             const unsigned char* src = raw + rs * (2 * RAW);
             unsigned char* dst = ring + slot * STAGE;
@@ -835,9 +841,10 @@ __device__ __forceinline__ void stage_volts(const CorrParams& P, unsigned char* 
   int rs = 0;
   uint32_t rpar = 1;
   int64_t n = 0;                                       // stages issued
+  int job = 0;
   bool ok = true;
   for (int64_t item = pair; item < P.total && ok; item += npairs) {
-    const CorrJob& J = *find_job(P, item);
+    const CorrJob& J = find_job(P, item, job);
     const int nt = J.nt, np = J.np, npol = J.a.npol, nch = J.nch;
     const int64_t jw = (item - J.item0) / J.a.nfreq;
     const int f = (int)(item - J.item0 - jw * J.a.nfreq), t0 = (int)(jw * J.a.n_int);
@@ -857,10 +864,7 @@ __device__ __forceinline__ void stage_volts(const CorrParams& P, unsigned char* 
         }
       }
   }
-  if (!ok) {
-    *abort_sm = 1;
-    atomicExch(P.err, FFTBF_ETIMEOUT);
-  }
+  if (!ok) corr_fail(P, abort_sm);
   // every copy issued must have landed before the CTA exits
   volatile int never = 0;
   for (int64_t i = n > NR ? n - NR : 0; i < n; ++i)
@@ -875,10 +879,10 @@ __device__ __forceinline__ void produce_direct(const CorrParams& P, unsigned cha
   const int k = (t & 7) + 8 * ((t >> 6) & 1), fb = (t >> 3) & 7;
   ring += (t & 7) * 16 + ((t >> 6) & 1) * LBO + fb * SBO;
   const uint32_t full0 = map_rank(tc::smem_u32(bars + FULL), 0);
-  int slot = 0, turn = 0;
+  int slot = 0, turn = 0, job = 0;
   uint32_t par = 1;
   for (int64_t item = pair; item < P.total; item += npairs) {
-    const CorrJob& J = *find_job(P, item);
+    const CorrJob& J = find_job(P, item, job);
     const BeamArgs& a = J.a;
     const int nt = J.nt, np = J.np, nsnap = a.n_int * a.npol, nyp = J.nyp, ny = J.ny, nx = a.nx;
     const uint8_t* begin = a.volts;
@@ -899,10 +903,7 @@ __device__ __forceinline__ void produce_direct(const CorrParams& P, unsigned cha
         for (int g = k; g - k < nsnap; g += KS) {
           if (turn == grp) {
             const bool ok = wait_pair(bars + EMPTY + slot, par, abort_sm);
-            if (!ok) {
-              *abort_sm = 1;
-              atomicExch(P.err, FFTBF_ETIMEOUT);
-            }
+            if (!ok) corr_fail(P, abort_sm);
             if (!__all_sync(0xffffffffu, ok)) return;
 #pragma unroll 1
             for (int b = 0; b < (hasb ? 2 : 1); ++b) {
@@ -972,10 +973,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(corr::NT, 1)
   cluster_sync();
   tc::fence_after_sync();
   const uint32_t tbase = taddr_sm;
-  auto fail = [&]() {
-    *abort_sm = 1;
-    atomicExch(P.err, FFTBF_ETIMEOUT);
-  };
+  auto fail = [&]() { corr_fail(P, abort_sm); };
   auto wait_one = [&](int bar, uint32_t parity) -> bool {
     if (wait_pair(bars + bar, parity, abort_sm)) return true;
     fail();
@@ -1003,10 +1001,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(corr::NT, 1)
       }
     };
     int64_t item = pair;
+    int job = 0;
     uint32_t ph = 0, iph = 0;                          // tile and item parities
     bool ok = true;
     while (item < P.total && ok) {
-      const CorrJob& J = *find_job(P, item);
+      const CorrJob& J = find_job(P, item, job);
       const JobRegs R{J.a.nx, J.ny, J.nyp, J.np, J.nt, J.a.mx, J.mode + (CPLX && !J.a.real_w ? 4 : 0)};
       const int nv = R.mx * R.ny;
       if (&J != last) {                                // weights in slot order, zeros between
@@ -1144,9 +1143,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(corr::NT, 1)
     int slot = 0;
     uint32_t par = 0, tph = 1;                         // tph: parity of the drained barrier
     int64_t tiles = 0;
+    int job = 0;
     bool ok = true;
     for (int64_t item = pair; item < P.total && ok; item += npairs) {
-      const CorrJob& J = *find_job(P, item);
+      const CorrJob& J = find_job(P, item, job);
       const int nt = J.nt, np = J.np, nsnap = J.a.n_int * J.a.npol;
       for (int I = 0; I < nt && ok; ++I)
         for (int Jc = I; Jc < nt && ok; ++Jc) {
@@ -1339,7 +1339,7 @@ bool corr_preferred(const BeamArgs& a) {
   return cov < per * nsnap;
 }
 
-int launch_beams_corr(const BeamArgs& a, int* err, int nsm, cudaStream_t st) {
+int launch_beams_corr(const BeamArgs& a, int nsm, cudaStream_t st) {
   CorrParams p{};
   if (!corr_make_job(a, &p.one) || !corr_sizes(&p.one, 1, &p.s))
     return set_error(FFTBF_EUNSUPPORTED, "lattice too large for the covariance kernel");
@@ -1347,8 +1347,40 @@ int launch_beams_corr(const BeamArgs& a, int* err, int nsm, cudaStream_t st) {
   if (rc != FFTBF_OK) return rc;
   p.total = p.one.nitems;
   p.njobs = 1;
-  p.err = err;
   return corr_launch(p, nsm, st);
+}
+
+// Cut a list of jobs (d_table: its device copy) into launches whose shared memory fits, usually
+// one, costliest items first, and number each launch's items.
+int corr_plan_jobs(std::vector<CorrJob>& jobs, const CorrJob* d_table, int* err,
+                   std::vector<CorrParams>* out) {
+  out->clear();
+  std::stable_sort(jobs.begin(), jobs.end(), [](const CorrJob& x, const CorrJob& y) {
+    return (double)x.np * x.np * x.nch > (double)y.np * y.np * y.nch;
+  });
+  for (size_t i = 0; i < jobs.size();) {
+    CorrParams p{};
+    size_t n = 1;
+    CorrSizes s;
+    if (!corr_sizes(&jobs[i], 1, &p.s))
+      return set_error(FFTBF_EUNSUPPORTED, "lattice too large for the covariance kernel");
+    while (i + n < jobs.size() && corr_sizes(&jobs[i], (int)n + 1, &s)) {
+      p.s = s;
+      ++n;
+    }
+    const int rc = corr_maps(&jobs[i], (int)n, p.s);
+    if (rc != FFTBF_OK) return rc;
+    for (size_t k = i; k < i + n; ++k) {
+      jobs[k].item0 = p.total;
+      p.total += jobs[k].nitems;
+    }
+    p.table = d_table + i;
+    p.njobs = (int)n;
+    p.err = err;
+    out->push_back(p);
+    i += n;
+  }
+  return FFTBF_OK;
 }
 
 }  // namespace fftbf

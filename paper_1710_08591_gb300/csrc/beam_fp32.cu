@@ -88,7 +88,7 @@ extern template int launch_fft_mx<16>(const BeamArgs&, int, int, cudaStream_t);
 int launch_beams_fp32(const BeamArgs& a, int nsm, cudaStream_t st) {
   if (a.nwin <= 0) return FFTBF_OK;
   if (a.err && !getenv_flag("FFTBF_FP32_GENERIC") && corr_preferred(a))
-    return launch_beams_corr(a, a.err, nsm, st);
+    return launch_beams_corr(a, nsm, st);
   if (fp32_n512_supported(a) && !getenv_flag("FFTBF_FP32_GENERIC"))
     return launch_beams_fp32_n512(a, nsm, st);
   if (fp32_warp_supported(a) && !getenv_flag("FFTBF_FP32_GENERIC"))

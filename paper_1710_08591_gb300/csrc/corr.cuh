@@ -29,15 +29,20 @@ struct CorrParams {
   const CorrJob* table; // a device table of njobs
   int njobs;
   int64_t total;        // work items
-  int* err;
+  int* err;             // error word, or null: those of the jobs' plans
   CorrSizes s;
 };
 
+// Fill a job; false where the kernel does not take the lattice.
 bool corr_make_job(const BeamArgs& a, CorrJob* J);
 bool corr_sizes(const CorrJob* jobs, int n, CorrSizes* out);
 int corr_maps(CorrJob* jobs, int n, const CorrSizes& s);
 int corr_launch(CorrParams& p, int nsm, cudaStream_t st);
+constexpr int kCorrSteps = 64;   // snapshots per operand stage
 bool corr_preferred(const BeamArgs& a);
-int launch_beams_corr(const BeamArgs& a, int* err, int nsm, cudaStream_t st);
+bool batch_cov(const fftbf_batch* bb, int i);   // plan i of the batch goes through it
+int launch_beams_corr(const BeamArgs& a, int nsm, cudaStream_t st);
+int corr_plan_jobs(std::vector<CorrJob>& jobs, const CorrJob* d_table, int* err,
+                   std::vector<CorrParams>* out);
 
 }  // namespace fftbf

@@ -8,7 +8,8 @@
 //   staging    admitted frames are copied host -> slot on a copy stream (one event each);
 //   ticks      whenever frames are staged and fewer than kTicks launches are in flight,
 //              every staged frame (up to 64) goes into ONE persistent launch of the batch
-//              kernel (one job per frame) on the next tick stream, which waits for the
+//              kernel (one job per frame; frames of lattices that take the covariance
+//              kernel in one launch of that) on the next tick stream, which waits for the
 //              frames' copy events; the beams are copied back to the caller's buffers on
 //              the same stream. Frames that arrive while ticks run join the next tick, so
 //              work from different arrivals overlaps on the device.
@@ -36,6 +37,7 @@
 #include <thread>
 #include <vector>
 
+#include "corr.cuh"
 #include "internal.cuh"
 
 namespace fftbf {
@@ -62,6 +64,9 @@ struct Tick {
   cudaEvent_t done = nullptr;
   BatchJob* d_jobs = nullptr;
   unsigned long long* d_counter = nullptr;
+  CorrJob* d_cjobs = nullptr;            // jobs of the covariance kernel and its error word
+  int* d_err = nullptr;
+  int* h_err = nullptr;
   std::vector<Frame> frames;
   bool busy = false;
 };
@@ -141,26 +146,50 @@ void fail(fftbf_server* sv, int rc) {
 int launch_tick(fftbf_server* sv, Tick& tk, int64_t* items_out) {
   NvtxRange nvtx("serve tick");
   const int n = (int)tk.frames.size();
-  std::vector<BatchJob> jobs(n);
-  int64_t total = 0;
+  std::vector<BatchJob> jobs;
+  std::vector<CorrJob> cjobs;
+  int64_t total = 0, items = 0;
   for (int k = 0; k < n; ++k) {
     const Frame& f = tk.frames[k];
     const fftbf_plan* p = sv->lattices[f.lattice];
-    BatchJob& J = jobs[k];
+    BatchJob J{};
     batch_fill_args(p, J.a);
     J.a.S = sv->S[f.lattice];
     unsigned char* slot = sv->arena + (size_t)f.slot * sv->slot_bytes;
     J.a.volts = slot;
     J.a.beams = reinterpret_cast<float*>(slot + sv->frame_off);
     J.a.nwin = 1;
-    J.variant = sv->V[f.lattice];
     J.nitems = p->nfreq;
+    items += J.nitems;
+    if (cudaStreamWaitEvent(tk.st, f.copied, 0) != cudaSuccess) return FFTBF_ECUDA;
+    if (batch_cov(sv->tuner, f.lattice)) {
+      CorrJob C;
+      corr_make_job(J.a, &C);
+      cjobs.push_back(C);
+      continue;
+    }
+    J.variant = sv->V[f.lattice];
     J.item0 = total;
     total += J.nitems;
-    if (cudaStreamWaitEvent(tk.st, f.copied, 0) != cudaSuccess) return FFTBF_ECUDA;
+    jobs.push_back(J);
   }
-  *items_out = total;
-  int rc = batch_launch_jobs(jobs.data(), n, tk.d_jobs, tk.d_counter, sv->smem, sv->grid, tk.st);
+  *items_out = items;
+  int rc = FFTBF_OK;
+  if (!cjobs.empty()) {
+    std::vector<CorrParams> launches;
+    rc = corr_plan_jobs(cjobs, tk.d_cjobs, tk.d_err, &launches);
+    if (rc == FFTBF_OK && cudaMemcpyAsync(tk.d_cjobs, cjobs.data(), sizeof(CorrJob) * cjobs.size(),
+                                          cudaMemcpyHostToDevice, tk.st) != cudaSuccess)
+      rc = FFTBF_ECUDA;
+    for (CorrParams& p : launches)
+      if (rc == FFTBF_OK) rc = corr_launch(p, sv->lattices[0]->nsm, tk.st);
+    if (rc == FFTBF_OK && cudaMemcpyAsync(tk.h_err, tk.d_err, sizeof(int), cudaMemcpyDeviceToHost,
+                                          tk.st) != cudaSuccess)
+      rc = FFTBF_ECUDA;
+  }
+  if (rc == FFTBF_OK && !jobs.empty())
+    rc = batch_launch_jobs(jobs.data(), (int)jobs.size(), tk.d_jobs, tk.d_counter, sv->smem,
+                           sv->grid, tk.st);
   for (int k = 0; k < n && rc == FFTBF_OK; ++k) {
     const Frame& f = tk.frames[k];
     unsigned char* slot = sv->arena + (size_t)f.slot * sv->slot_bytes;
@@ -253,6 +282,7 @@ void run_scheduler(fftbf_server* sv) {
       const auto now = Clock::now();
       std::lock_guard<std::mutex> lk(sv->mu);
       if (q != cudaSuccess && sv->error == FFTBF_OK) sv->error = FFTBF_ECUDA;
+      if (*k.h_err && sv->error == FFTBF_OK) sv->error = *k.h_err;
       for (const Frame& f : k.frames) {
         record_done(sv, f.ticket, std::chrono::duration<double, std::milli>(now - f.t_submit).count());
         sv->free_slots.push_back(f.slot);
@@ -323,6 +353,11 @@ fftbf_server* fftbf_server_create(fftbf_plan* const* lattices, int n, int64_t hb
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&sv->ticks[t].done, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMalloc(&sv->ticks[t].d_jobs, sizeof(BatchJob) * kJobsPerTick);
     if (e == cudaSuccess) e = cudaMalloc(&sv->ticks[t].d_counter, sizeof(unsigned long long));
+    if (e == cudaSuccess) e = cudaMalloc(&sv->ticks[t].d_cjobs, sizeof(CorrJob) * kJobsPerTick);
+    if (e == cudaSuccess) e = cudaMalloc(&sv->ticks[t].d_err, sizeof(int));
+    if (e == cudaSuccess) e = cudaMemset(sv->ticks[t].d_err, 0, sizeof(int));
+    if (e == cudaSuccess) e = cudaMallocHost(&sv->ticks[t].h_err, sizeof(int));
+    if (e == cudaSuccess) *sv->ticks[t].h_err = 0;
   }
   if (e != cudaSuccess) {
     cuda_error(e, "fftbf_server_create");
@@ -429,6 +464,9 @@ void fftbf_server_destroy(fftbf_server* sv) {
     if (t.done) cudaEventDestroy(t.done);
     cudaFree(t.d_jobs);
     cudaFree(t.d_counter);
+    cudaFree(t.d_cjobs);
+    cudaFree(t.d_err);
+    cudaFreeHost(t.h_err);
     if (t.st) cudaStreamDestroy(t.st);
   }
   if (sv->copy_st) {

@@ -106,3 +106,64 @@ def test_constant_input_is_exact(monkeypatch):
     rest = got.copy()
     rest[0, 0] = 0
     assert rest.min() >= 0 and rest.max() <= 1e-12 * got[0, 0]
+
+
+def _batch(arrays, n_int, nwin, stream=None):
+    plans = [fb.plan_create(*s, 2, v.shape[1], n_int, weights=w)
+             for s, v, w in arrays]
+    dvs = [torch.from_numpy(np.ascontiguousarray(v).reshape(-1)).cuda() for _, v, _ in arrays]
+    outs = [torch.full((nwin, v.shape[1], s[2], s[3]), float("nan"), device="cuda") for s, v, _ in arrays]
+    with fb.batch_create(plans) as b:
+        for _ in range(2):
+            fb.batch_execute(b, dvs, nwin * n_int, outs, stream)
+        torch.cuda.synchronize()
+    for p in plans:
+        fb.plan_sync(p)
+        p.close()
+    return [o.cpu().numpy() for o in outs]
+
+
+@pytest.mark.parametrize("n_int", [50, 320])
+def test_batch_of_covariance_and_fft_arrays(n_int):
+    """100 snapshots per window: only the 8x64 arrays take the covariance; 640: all do, real
+    and complex weights in one launch. Every array matches the oracle and is bit-identical
+    alone and in the mix, captured or not."""
+    nwin = 2
+    shapes = [(4, 256, 4, 512), (8, 64, 8, 128), (16, 16, 16, 32), (2, 512, 2, 1024), (1, 1024, 1, 2048),
+              (3, 128, 3, 256)]
+    arrays = []
+    for k, s in enumerate(shapes):
+        v, w = make_case(*s, 2, 1 + k % 3, n_int * nwin, n_int, weights="random" if k % 2 else "half_sine",
+                         seed=60 + k)
+        arrays.append((s, v, w))
+    mix = _batch(arrays, n_int, nwin, torch.cuda.Stream())
+    plain = _batch(arrays, n_int, nwin)
+    for k, ((s, v, w), g) in enumerate(zip(arrays, mix)):
+        ref = oracle_beams(v, w, *s, 2, v.shape[1], n_int)
+        assert rel_err_per_beam(g, ref).max() <= TOL_BEAM, s
+        assert np.array_equal(g, plain[k]), s
+        assert np.array_equal(g, _batch([arrays[k]], n_int, nwin)[0]), s
+
+
+def test_server_frames_through_the_covariance():
+    """Frames of 320 samples x 2 polarisations on two lattices: the server's beams are those of
+    a batch of the frame alone and match the oracle."""
+    n_int, nf = 320, 2
+    shapes = [(8, 64, 8, 128), (4, 256, 4, 512)]
+    frames, outs = [], []
+    plans = [fb.plan_create(*s, 2, nf, n_int) for s in shapes]
+    with fb.server_create(plans, 64 << 20) as sv:
+        for k in range(6):
+            s = shapes[k % 2]
+            v, _ = make_case(*s, 2, nf, n_int, n_int, seed=200 + k)
+            frames.append(v)
+            outs.append(np.full((nf, s[2], s[3]), np.nan, np.float32))
+            fb.server_submit(sv, k % 2, v.reshape(-1), outs[-1])
+        fb.server_wait(sv)
+    for k, (v, o) in enumerate(zip(frames, outs)):
+        s = shapes[k % 2]
+        ref = oracle_beams(v, None, *s, 2, nf, n_int)
+        assert rel_err_per_beam(o[None], ref).max() <= TOL_BEAM
+        assert np.array_equal(o[None], _batch([(s, v, None)], n_int, 1)[0])
+    for p in plans:
+        p.close()
