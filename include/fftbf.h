@@ -60,8 +60,9 @@ enum fftbf_precision {
                               and transformed once per window in two-float FP32) */
   FFTBF_PREC_TC_FP16 = 1, /* tensor-core GEMM stages, FP16 operands, FP32 accumulate */
   FFTBF_PREC_TC_BF16 = 2, /* tensor-core GEMM stages, BF16 operands, FP32 accumulate */
-  FFTBF_PREC_TC_FP16X3 = 3 /* tensor-core GEMM stages on split FP16 operands (hi + lo,
-                              three products per stage), FP32 accumulate: FP32 accuracy */
+  FFTBF_PREC_TC_FP16X3 = 3 /* FP32 accuracy on the tensor cores: GEMM stages on split FP16
+                              operands (hi + lo, three products per stage, FP32 accumulate),
+                              or for windows of many snapshots the covariance of FP32 */
 };
 
 /*
@@ -90,7 +91,8 @@ fftbf_plan* fftbf_plan_create(int nx, int ny, int pad_x, int pad_y, int npol, in
  * removes the scale from the result. FFTBF_PREC_TC_FP16X3 splits every operand into an
  * FP16 value and its FP16 residual (hi + lo) and forms each stage as hi*hi + hi*lo +
  * lo*hi in FP32, so the result has FP32 accuracy (the dropped lo*lo term is ~2^-22 of
- * each product). On the 4x256 lattice with 16-byte aligned voltages the FP16 and BF16
+ * each product); windows of many snapshots take the covariance route of FFTBF_PREC_FP32,
+ * whose sums are exact. On the 4x256 lattice with 16-byte aligned voltages the FP16 and BF16
  * forms run a kernel that folds the E-W DFT into the first stage and keeps the second
  * stage's operand in tensor memory; the environment variable FFTBF_TC_KERNEL=ws selects
  * the pair-wise kernel (E-W DFT on the CUDA cores) instead and FFTBF_TC_KERNEL=serial the

@@ -305,7 +305,7 @@ __device__ __forceinline__ int tile_cols(int np, int J) {
 struct JobRegs { int nx, ny, nyp, np, nt, mx, mode; };
 
 struct Lay {                             // shared-memory offsets (bytes)
-  int ring, raw, w, v, stg, sl, total;
+  int ring, raw, w, v, stg, sl, tab, total;
 };
 __host__ __device__ inline Lay lay_of(const CorrSizes& s) {
   Lay L;
@@ -317,6 +317,7 @@ __host__ __device__ inline Lay lay_of(const CorrSizes& s) {
   L.v = take(s.vlen * 16);
   L.stg = take(s.stg * 8 * 4);           // 8 warps; also the transform's buffer
   L.sl = take(s.slice * 8 * 4);
+  L.tab = take(s.tab * 16);
   L.total = o;
   return L;
 }
@@ -633,6 +634,9 @@ __device__ __forceinline__ void corr_combine_blocks(const JobRegs& J, int row0, 
   }
 }
 
+// Entries of a twiddle table that a transform of n reads: half of them where n is a power of two.
+__host__ __device__ inline int tw_len(int n) { return (n & (n - 1)) == 0 && n > 1 ? n >> 1 : n; }
+
 // ---- transform of an item's V to beams (256 threads of each CTA of the pair; the first takes the
 // even pairs of E-W beams, the second the odd ones): over kappa in
 // place when mx is a power of two (decimation in frequency: E-W beam A ends in row brev(A)), by
@@ -640,10 +644,10 @@ __device__ __forceinline__ void corr_combine_blocks(const JobRegs& J, int row0, 
 // (their spectra are real): z = H_A0 + i H_A1 with H_A[m] the Hermitian part of the sum of
 // lambda = m (mod my).
 __device__ void corr_beams(const CorrJob& J, int64_t item, int rank, float* v, int nv, float4* z,
-                           int tid) {
+                           const float4* tw, int tid) {
   const BeamArgs& a = J.a;
   const int ny = J.ny, mx = a.mx, my = a.my;
-  const float4 *tw = a.cw, *ew = a.cw + my;            // exp(-2 pi i k / my), exp(-2 pi i k / mx)
+  const float4* ew = tw + tw_len(my);                  // exp(-2 pi i k / mx), after exp(-2 pi i k / my)
   const int np2 = ((mx + 1) / 2 - rank + 1) / 2;       // pairs of this CTA: u = 2 i + rank
   if (np2 <= 0) return;
   auto log2_of = [](int n) { return 31 - __clz(n); };
@@ -723,22 +727,15 @@ __device__ void corr_beams(const CorrJob& J, int64_t item, int rank, float* v, i
   }
   bar_epi();
   if (pow2y) {
-    // in place, decimation in time; the twiddle of a thread's first butterfly of the next stage
-    // is loaded before the barrier
-    auto twiddle = [&](int o, int st) { return tw[(o & (my >> 1) - 1 & (1 << st) - 1) << (lgy - 1 - st)]; };
-    float4 w = lgy ? twiddle(tid, 0) : make_float4(1.f, 0.f, 0.f, 0.f);
-    for (int st = 0; st < lgy; ++st) {
+    for (int st = 0; st < lgy; ++st) {                 // in place, decimation in time
       const int half = 1 << st;
-      const float4 next = st + 1 < lgy ? twiddle(tid, st + 1) : w;
       for (int o = tid; o < np2 * (my >> 1); o += EPI) {
         const int u = o >> (lgy - 1), b = o & ((my >> 1) - 1);
         const int k = b & (half - 1), i0 = u * my + ((b >> st) << (st + 1)) + k;
-        if (o != tid) w = twiddle(o, st);
-        const Cdd x = zget(i0), y = dd_cmul(zget(i0 + half), w);
+        const Cdd x = zget(i0), y = dd_cmul(zget(i0 + half), tw[k << (lgy - 1 - st)]);
         zput(i0, dd_add(x, y));
         zput(i0 + half, dd_sub(x, y));
       }
-      w = next;
       bar_epi();
     }
   }
@@ -989,6 +986,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(corr::NT, 1)
     float* vv = reinterpret_cast<float*>(smem + Y.v);
     float* stg = reinterpret_cast<float*>(smem + Y.stg);
     float* sl = reinterpret_cast<float*>(smem + Y.sl);
+    float4* tab = reinterpret_cast<float4*>(smem + Y.tab);
     const int wslots = P.s.wslots;
     const uint32_t rf = map_rank(tc::smem_u32(bars + RF), 0), imf = map_rank(tc::smem_u32(bars + IF), 0);
     const CorrJob* last = nullptr;
@@ -1017,6 +1015,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(corr::NT, 1)
           ws[s] = w.x;
           if (CPLX) ws[wslots + s] = w.y;
         }
+        const int ty = tw_len(J.a.my), tx = tw_len(J.a.mx);
+        for (int i = tid; i < ty + tx; i += EPI) tab[i] = J.a.cw[i < ty ? i : J.a.my + i - ty];
         last = &J;
         zero_rows();
         bar_epi();
@@ -1113,7 +1113,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(corr::NT, 1)
       }
       bar_epi();
       if (tid == 0) arrive_release_cluster(map_rank(tc::smem_u32(bars + PE), rank ^ 1));
-      corr_beams(J, item - J.item0, (int)rank, u, nv, reinterpret_cast<float4*>(u + 4 * nv), tid);
+      corr_beams(J, item - J.item0, (int)rank, u, nv, reinterpret_cast<float4*>(u + 4 * nv), tab, tid);
       if (tid == 0) {
         ok = wait_pair<true>(bars + PE, iph, abort_sm);   // the other CTA has read this one's V
         if (!ok) fail();
@@ -1246,6 +1246,7 @@ bool corr_sizes(const CorrJob* jobs, int n, CorrSizes* out) {
     s.vlen = std::max(s.vlen, j.a.mx * j.ny);
     s.stg = std::max({s.stg, c * stg_floats(G, CR), (4 * j.a.mx * j.ny + ((j.a.mx + 1) / 2 + 1) / 2 * j.a.my * 4 + 7) / 8});
     s.slice = std::max(s.slice, 2 * slice_floats(G, CR));
+    s.tab = std::max(s.tab, tw_len(j.a.my) + tw_len(j.a.mx));
   }
   s.stg = (s.stg + 3) & ~3;
   const int most = 227 * 1024 - 1024;                  // static shared memory: the barriers
@@ -1313,10 +1314,11 @@ int corr_launch(CorrParams& p, int nsm, cudaStream_t st) {
 //               times that where the voltages cannot come by TMA;
 //   transform   us per snapshot and 1000 beams: 0.8 the 512-beam kernels (4x256: 827 us at 512),
 //               0.6 the 32-beam kernel, 1.1 those of 1024 and 2048 beams, 1.9 the other FFT
-//               kernels (8x64: 980 us at 512); the direct DFT 1.0 for every N-S feed.
+//               kernels (8x64: 980 us at 512); the direct DFT 1.0 for every N-S feed. The
+//               split-FP16 kernel (split) 1.3 (4x256: 2060 us at 768).
 // So 4x256 changes over near 300 snapshots, 8x64 near 90, 16x16 near 400. Only the plan's sizes
 // enter, never the number of windows or the pointer: a window's beams do not depend on its call.
-bool corr_preferred(const BeamArgs& a) {
+bool corr_preferred(const BeamArgs& a, bool split) {
   CorrJob j;
   CorrSizes s;
   if (!corr_make_job(a, &j) || !corr_sizes(&j, 1, &s)) return false;
@@ -1332,7 +1334,8 @@ bool corr_preferred(const BeamArgs& a) {
   const double fixed = (34.0 * tiles + 55.0) * (a.real_w ? 1.0 : 1.4);
   const double cov = std::max(fixed, 0.6 * fixed + 0.021 * (j.ny % 16 == 0 && corr::KS % a.npol == 0 ? 1 : 3) * units * nsnap);
   double per;                                          // us per snapshot
-  if (fp32_n512_supported(a)) per = 0.8e-3 * nout;
+  if (split) per = 1.3e-3 * nout;
+  else if (fp32_n512_supported(a)) per = 0.8e-3 * nout;
   else if (fp32_warp_supported(a)) per = (a.my == 32 ? 0.6e-3 : a.my >= 1024 ? 1.1e-3 : 1.9e-3) * nout;
   else if (fp32_fft_supported(a.mx, a.my)) per = 1.9e-3 * std::max<double>(nout, j.nant);
   else per = 1e-3 * nout * a.nyf;

@@ -20,7 +20,7 @@ struct CorrJob {
 };
 struct CorrSizes {      // shared-memory sizes, the largest over the launch's jobs
   int ns, nr;           // operand stages, staged voltage tiles
-  int wslots, vlen, stg, slice;
+  int wslots, vlen, stg, slice, tab;
   int cplx;             // some weights are complex
   int tma;              // every job's voltages are staged by TMA
 };
@@ -39,7 +39,8 @@ bool corr_sizes(const CorrJob* jobs, int n, CorrSizes* out);
 int corr_maps(CorrJob* jobs, int n, const CorrSizes& s);
 int corr_launch(CorrParams& p, int nsm, cudaStream_t st);
 constexpr int kCorrSteps = 64;   // snapshots per operand stage
-bool corr_preferred(const BeamArgs& a);
+// Whether it beats the transform of every snapshot (split: the split-FP16 kernel).
+bool corr_preferred(const BeamArgs& a, bool split = false);
 bool batch_cov(const fftbf_batch* bb, int i);   // plan i of the batch goes through it
 int launch_beams_corr(const BeamArgs& a, int nsm, cudaStream_t st);
 int corr_plan_jobs(std::vector<CorrJob>& jobs, const CorrJob* d_table, int* err,

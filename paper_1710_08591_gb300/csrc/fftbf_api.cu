@@ -9,6 +9,7 @@
 #include <new>
 #include <string>
 
+#include "corr.cuh"
 #include "internal.cuh"
 
 namespace fftbf {
@@ -215,6 +216,8 @@ int fftbf_execute(fftbf_plan* p, const uint8_t* volts, int64_t T, float* beams, 
   int rc;
   if (p->precision == FFTBF_PREC_FP32) {
     rc = launch_beams_fp32(a, p->nsm, st);
+  } else if (p->precision == FFTBF_PREC_TC_FP16X3 && corr_preferred(a, true)) {
+    rc = launch_beams_corr(a, p->nsm, st);             // FP32 accuracy on the tensor cores, faster
   } else {
     TcArgs ta{};
     ta.b = a;
