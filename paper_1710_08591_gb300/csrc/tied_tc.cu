@@ -7,11 +7,11 @@
 // keeps FP32 accuracy; e scales every weight row and every beam row so that its largest
 // magnitude lies in [2^14, 2^15) (inside the FP16 range, with the residuals normal), and the
 // epilogue divides by 2^(e_s + e_j) exactly. Both split operands are stored in global
-// memory already cut into 16 KB tiles (128 rows x 64 beams, the canonical K-major layout,
-// zero rows past the ends). A CTA computes 128 pointings x 128 windows of one channel: one
-// thread stages each K chunk as four bulk copies completing on a full-mbarrier (three
+// memory already cut into tiles (128 pointings or TN windows x 64 beams, the canonical K-major
+// layout, zero rows past the ends). A CTA computes 128 pointings x TN windows of one channel: one
+// thread stages each K chunk as four bulk copies completing on a full-mbarrier (two or three
 // stages), issues its MMAs and commits them to the stage's empty-mbarrier; one TMEM
-// accumulator of 128 columns per E-W beam used by the tile's pointings, and each pointing
+// accumulator of TN columns per E-W beam used by the tile's pointings, and each pointing
 // (TMEM lane) reads its own beam's accumulator. Every wait is bounded; a timeout sets the
 // plan's error word.
 #include <cuda_fp16.h>
@@ -26,14 +26,23 @@
 namespace fftbf {
 
 namespace ttc {
-constexpr int TM = 128, TN = 128, KC = 64;     // pointings, windows, beams per K chunk
+constexpr int TM = 128, KC = 64;               // pointings, beams per K chunk
 constexpr int LBO = 128, SBO = 1024;           // canonical K-major tile: 8 K blocks per row group
 constexpr int TILE = TM * KC * 2;              // bytes of one 128 x 64 FP16 tile
-constexpr int STAGE = 4 * TILE;                // W hi, W lo, P hi, P lo
 constexpr int NT = 256;                        // warps w and w + 4 share TMEM lane quarter w % 4
-constexpr int NS = 3;                          // staging buffers
 constexpr int MAXA = 4;                        // E-W beams (one accumulator each)
-constexpr uint32_t TMEM_COLS = 512;
+// By windows per CTA TN: 128 in general; 64 for calls of at most 64 windows, where half of the MMA
+// columns and of the beam tiles would be padding, and where two CTAs then fit on an SM, so that
+// one's set-up and scattered stores run under the other's products. 256 channels x 2048 pointings
+// x 64 windows, whose split weights are 1.07 GB per call: 635 -> 415 us per call with the prep
+// kernel below.
+template <int TN> struct Cfg {
+  static constexpr int PT = TN * KC * 2;       // bytes of one TN x 64 beam tile
+  static constexpr int STAGE = 2 * TILE + 2 * PT;   // W hi, W lo, P hi, P lo
+  static constexpr int NS = TN == 64 ? 2 : 3;  // staging buffers
+  static constexpr int CTAS = TN == 64 ? 2 : 1;
+  static constexpr uint32_t TMEM_COLS = MAXA * TN;
+};
 constexpr uint64_t WAIT_NS = 1000000000ull;
 }  // namespace ttc
 
@@ -100,47 +109,98 @@ __global__ void tied_tc_table_kernel(const float* __restrict__ wx, const float* 
   }
 }
 
-// Beam rows P[j, f, A, :] split the same way (per call), in tiles per (channel, E-W beam) of
-// 128 windows (zero rows past nwin); exponents at pe[(j nfreq + f) mx + A].
+// x 2^e, rounded once as ldexpf does.
+__device__ __forceinline__ float scale_pow2(float x, int e) {
+  return e >= -126 && e <= 127 ? x * __int_as_float((127 + e) << 23) : ldexpf(x, e);
+}
+
+// Beam rows P[j, f, A, :] split the same way (per call), in tiles per (channel, E-W beam) of TN
+// windows (zero rows past nwin); exponents at pe[(j nfreq + f) mx + A]. A warp takes eight windows,
+// lane (g, r) eight beams of window r at a time: 128 contiguous bytes are read per window, and the
+// eight windows' 16-byte pieces of one K block are the 128 bytes of a core matrix, so every store
+// of the warp is 512 contiguous bytes (a row per warp wrote 16-byte pieces 128 bytes apart).
+template <int TN>
 __global__ void tied_tc_prep_kernel(const float* __restrict__ P, int64_t nwin, int nfreq, int mx,
-                                    int my, __half* ph, __half* pl, int* pe) {
-  const int lane = threadIdx.x & 31;
-  const int ntj = (int)((nwin + ttc::TN - 1) / ttc::TN), kcs = my / ttc::KC;
-  const int64_t per_fa = (int64_t)ntj * ttc::TN;
-  const int64_t nrows = (int64_t)nfreq * mx * per_fa;
+                                    int my, __half* ph, __half* pl, int* pe, int vec) {
+  const int lane = threadIdx.x & 31, r = lane & 7, g = lane >> 3;
+  const int ntj = (int)((nwin + TN - 1) / TN), kcs = my / ttc::KC;
+  const int64_t per_fa = (int64_t)ntj * (TN / 8);      // groups of eight windows
+  const int64_t ngrp = (int64_t)nfreq * mx * per_fa;
   const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t rp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); rp < nrows; rp += nw) {
-    const int64_t fa = rp / per_fa;                 // f mx + A
-    const int64_t j = rp - fa * per_fa;
+  for (int64_t gp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); gp < ngrp; gp += nw) {
+    const int64_t fa = gp / per_fa;                    // f mx + A
+    const int64_t j8 = gp - fa * per_fa, j = 8 * j8 + r;
     const int f = (int)(fa / mx), A = (int)(fa - (int64_t)f * mx);
-    const int64_t tile0 = (fa * ntj + (j >> 7)) * kcs;
-    const float* x = j < nwin ? P + ((j * nfreq + f) * mx + A) * my : nullptr;
-    const int e = split_row_tiled(x, 1.f, my, ph, pl, tile0, (int)(j & 127), lane);
-    if (x && lane == 0) pe[(j * nfreq + f) * mx + A] = e;
+    const bool live = j < nwin;
+    const float* x = P + ((live ? j * nfreq + f : 0) * mx + A) * my + 8 * g;
+    auto load = [&](int k, float (&v)[8]) {
+      if (vec) {
+        const float4 a = *reinterpret_cast<const float4*>(x + k), b = *reinterpret_cast<const float4*>(x + k + 4);
+        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+        v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+      } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = x[k + i];
+      }
+    };
+    float m = 0.f;
+    if (live)
+#pragma unroll 4
+      for (int k = 0; k < my; k += 32) {
+        float v[8];
+        load(k, v);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) m = fmaxf(m, fabsf(v[i]));
+      }
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 8));
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
+    const int e = split_exp(m);
+    // this group's rows in the tile of chunk 0 (halves)
+    const int jt = (int)(8 * j8 / TN), row = (int)(8 * j8 - (int64_t)jt * TN);
+    const int64_t base = (fa * ntj + jt) * kcs * (TN * ttc::KC) + (row >> 3) * (ttc::SBO / 2) + lane * 8;
+#pragma unroll 4
+    for (int k = 0; k < my; k += 32) {
+      float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      if (live) load(k, v);
+      __half2 h[4], l[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float a = scale_pow2(v[2 * i], e), b = scale_pow2(v[2 * i + 1], e);
+        h[i] = __halves2half2(__float2half_rn(a), __float2half_rn(b));
+        l[i] = __halves2half2(__float2half_rn(a - __low2float(h[i])), __float2half_rn(b - __high2float(h[i])));
+      }
+      const int64_t o = base + (int64_t)(k >> 6) * (TN * ttc::KC) + ((k & 63) >> 3) * (ttc::LBO / 2);
+      *reinterpret_cast<uint4*>(ph + o) = *reinterpret_cast<const uint4*>(h);
+      *reinterpret_cast<uint4*>(pl + o) = *reinterpret_cast<const uint4*>(l);
+    }
+    if (live && g == 0) pe[(j * nfreq + f) * mx + A] = e;
   }
 }
 
-__global__ void __launch_bounds__(ttc::NT, 1) tied_tc_kernel(
+template <int TN>
+__global__ void __launch_bounds__(ttc::NT, ttc::Cfg<TN>::CTAS) tied_tc_kernel(
     const __half* __restrict__ wyh, const __half* __restrict__ wyl, const int* __restrict__ wye,
     const int* __restrict__ wa, const int* __restrict__ perm, const __half* __restrict__ ph,
     const __half* __restrict__ pl, const int* __restrict__ pe, float* __restrict__ out,
     int64_t nwin, int nfreq, int n_tied, int mx, int my, int* err) {
+  using C = ttc::Cfg<TN>;
+  constexpr int NS = C::NS, STAGE = C::STAGE, PT = C::PT;
   extern __shared__ __align__(1024) unsigned char smem_t[];
-  __shared__ uint64_t full[ttc::NS], empty[ttc::NS];
+  __shared__ uint64_t full[NS], empty[NS];
   __shared__ uint32_t taddr;
   __shared__ int s_mask;
-  __shared__ int s_pe[ttc::MAXA][ttc::TN];
+  __shared__ int s_pe[ttc::MAXA][TN];
   const int tid = threadIdx.x, warp = tid >> 5;
   const int f = blockIdx.z;
   const int s0 = blockIdx.x * ttc::TM;
-  const int64_t j0 = (int64_t)blockIdx.y * ttc::TN;
+  const int64_t j0 = (int64_t)blockIdx.y * TN;
   const int64_t fs0 = (int64_t)f * n_tied;
   if (warp == 0) {
-    tc::tmem_alloc(&taddr, ttc::TMEM_COLS);
+    tc::tmem_alloc(&taddr, C::TMEM_COLS);
     tc::tmem_relinquish();
   }
   if (tid == 0) {
-    for (int i = 0; i < ttc::NS; ++i) {
+    for (int i = 0; i < NS; ++i) {
       tc::mbar_init(&full[i], 1);
       tc::mbar_init(&empty[i], 1);
     }
@@ -163,8 +223,8 @@ __global__ void __launch_bounds__(ttc::NT, 1) tied_tc_kernel(
       ++nact;
     }
   // exponents of the tile's windows, per E-W beam in use
-  for (int i = tid; i < nact * ttc::TN; i += ttc::NT) {
-    const int ai = i / ttc::TN, jj = i - ai * ttc::TN;
+  for (int i = tid; i < nact * TN; i += ttc::NT) {
+    const int ai = i / TN, jj = i - ai * TN;
     int A = 0;
     for (int a = 0, c = -1; a < mx; ++a)
       if ((mask >> a) & 1 && ++c == ai) A = a;
@@ -177,41 +237,41 @@ __global__ void __launch_bounds__(ttc::NT, 1) tied_tc_kernel(
   const uint32_t tbase = taddr;
   const int kcs = my / ttc::KC;
   const int total = nact * kcs;
-  const uint32_t idesc = tc::idesc_f16(ttc::TM, ttc::TN, false);
+  const uint32_t idesc = tc::idesc_f16(ttc::TM, TN, false);
   // Thread 0 runs the pipeline: chunk t = (E-W beam in use number t / kcs, K chunk t % kcs)
-  // goes to stage t % NS as four 16 KB bulk copies completing on full[stage]; its MMAs
+  // goes to stage t % NS as four bulk copies completing on full[stage]; its MMAs
   // commit to empty[stage], after which the stage takes chunk t + NS. The other threads wait
   // at the CTA barrier. Every wait is bounded.
   __shared__ int s_ok;
   if (tid == 0) {
     bool ok = true;
     const int nts = (n_tied + ttc::TM - 1) / ttc::TM;
-    const int ntj = (int)((nwin + ttc::TN - 1) / ttc::TN);
+    const int ntj = (int)((nwin + TN - 1) / TN);
     const int64_t wt0 = ((int64_t)f * nts + blockIdx.x) * kcs;   // first weight tile
     auto issue = [&](int t) {
-      const int st = t % ttc::NS;
-      unsigned char* stg = smem_t + st * ttc::STAGE;
+      const int st = t % NS;
+      unsigned char* stg = smem_t + st * STAGE;
       const int ai = t / kcs, kc = t - ai * kcs;
       int A = 0;
       for (int a = 0, c = -1; a < mx; ++a)
         if ((mask >> a) & 1 && ++c == ai) A = a;
       const int64_t pt = (((int64_t)f * mx + A) * ntj + blockIdx.y) * kcs + kc;
       const int64_t wt = wt0 + kc;
-      tc::mbar_arrive_expect_tx(&full[st], (uint32_t)ttc::STAGE);
+      tc::mbar_arrive_expect_tx(&full[st], (uint32_t)STAGE);
       tc::bulk_g2s(stg, wyh + wt * (ttc::TILE / 2), ttc::TILE, &full[st]);
       tc::bulk_g2s(stg + ttc::TILE, wyl + wt * (ttc::TILE / 2), ttc::TILE, &full[st]);
-      tc::bulk_g2s(stg + 2 * ttc::TILE, ph + pt * (ttc::TILE / 2), ttc::TILE, &full[st]);
-      tc::bulk_g2s(stg + 3 * ttc::TILE, pl + pt * (ttc::TILE / 2), ttc::TILE, &full[st]);
+      tc::bulk_g2s(stg + 2 * ttc::TILE, ph + pt * (PT / 2), PT, &full[st]);
+      tc::bulk_g2s(stg + 2 * ttc::TILE + PT, pl + pt * (PT / 2), PT, &full[st]);
     };
-    for (int t = 0; t < ttc::NS && t < total; ++t) issue(t);
+    for (int t = 0; t < NS && t < total; ++t) issue(t);
     for (int t = 0; t < total && ok; ++t) {
-      const int st = t % ttc::NS;
-      const uint32_t par = (uint32_t)((t / ttc::NS) & 1);
+      const int st = t % NS;
+      const uint32_t par = (uint32_t)((t / NS) & 1);
       ok = tc::mbar_wait(&full[st], par, ttc::WAIT_NS);
       if (!ok) break;
       tc::fence_after_sync();
-      const uint32_t sa = tc::smem_u32(smem_t + st * ttc::STAGE);
-      const uint32_t d = tbase + (uint32_t)((t / kcs) * ttc::TN);
+      const uint32_t sa = tc::smem_u32(smem_t + st * STAGE);
+      const uint32_t d = tbase + (uint32_t)((t / kcs) * TN);
       const int kc = t % kcs;
 #pragma unroll
       for (int ks = 0; ks < ttc::KC / 16; ++ks) {
@@ -219,7 +279,7 @@ __global__ void __launch_bounds__(ttc::NT, 1) tied_tc_kernel(
         const uint64_t dwh = tc::smem_desc(sa + ko, ttc::LBO, ttc::SBO);
         const uint64_t dwl = tc::smem_desc(sa + ttc::TILE + ko, ttc::LBO, ttc::SBO);
         const uint64_t dph = tc::smem_desc(sa + 2 * ttc::TILE + ko, ttc::LBO, ttc::SBO);
-        const uint64_t dpl = tc::smem_desc(sa + 3 * ttc::TILE + ko, ttc::LBO, ttc::SBO);
+        const uint64_t dpl = tc::smem_desc(sa + 2 * ttc::TILE + PT + ko, ttc::LBO, ttc::SBO);
         tc::mma_f16(d, dwh, dph, idesc, (kc > 0 || ks > 0) ? 1u : 0u);
         tc::mma_f16(d, dwh, dpl, idesc, 1u);
         tc::mma_f16(d, dwl, dph, idesc, 1u);
@@ -227,14 +287,14 @@ __global__ void __launch_bounds__(ttc::NT, 1) tied_tc_kernel(
       tc::mma_commit(&empty[st]);
       // refill the stage of chunk t - 1 once its MMAs are done
       const int tp = t - 1;
-      if (tp >= 0 && tp + ttc::NS < total) {
-        ok = tc::mbar_wait(&empty[tp % ttc::NS], (uint32_t)((tp / ttc::NS) & 1), ttc::WAIT_NS);
-        if (ok) issue(tp + ttc::NS);
+      if (tp >= 0 && tp + NS < total) {
+        ok = tc::mbar_wait(&empty[tp % NS], (uint32_t)((tp / NS) & 1), ttc::WAIT_NS);
+        if (ok) issue(tp + NS);
       }
     }
     if (ok && total > 0) {                          // the last commit covers every MMA
       const int tl = total - 1;
-      ok = tc::mbar_wait(&empty[tl % ttc::NS], (uint32_t)((tl / ttc::NS) & 1), ttc::WAIT_NS);
+      ok = tc::mbar_wait(&empty[tl % NS], (uint32_t)((tl / NS) & 1), ttc::WAIT_NS);
     }
     s_ok = ok ? 1 : 0;
   }
@@ -243,13 +303,13 @@ __global__ void __launch_bounds__(ttc::NT, 1) tied_tc_kernel(
   const bool ok = s_ok != 0;
   tc::fence_after_sync();
   if (ok && total > 0) {
-    // warp w reads TMEM lanes 32 (w % 4) .. + 31 (its pointings) and windows 64 (w / 4) .. + 63
+    // warp w reads TMEM lanes 32 (w % 4) .. + 31 (its pointings) and half w / 4 of the windows
     const uint32_t lane_off = (uint32_t)(32 * (warp & 3)) << 16;
     const int dst_s = srow ? perm[fs0 + s] : 0;
-    for (int c = 2 * (warp >> 2); c < 2 * (warp >> 2) + 2; ++c) {
+    for (int c = TN / 64 * (warp >> 2); c < TN / 64 * (warp >> 2) + TN / 64; ++c) {
       for (int a2 = 0; a2 < nact; ++a2) {
         uint32_t r[32];
-        tc::tmem_ld32(tbase + lane_off + (uint32_t)(a2 * ttc::TN + 32 * c), r);
+        tc::tmem_ld32(tbase + lane_off + (uint32_t)(a2 * TN + 32 * c), r);
         tc::tmem_wait_ld();
         if (a2 == my_ai && srow) {
 #pragma unroll
@@ -271,7 +331,7 @@ __global__ void __launch_bounds__(ttc::NT, 1) tied_tc_kernel(
   }
   tc::fence_before_sync();
   __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tbase, ttc::TMEM_COLS);
+  if (warp == 0) tc::tmem_dealloc(tbase, C::TMEM_COLS);
 }
 
 // ------------------------------------------------------------------------------ host --
@@ -320,12 +380,13 @@ int tied_tc_build(TiedTables& tt, int64_t nuv, int mx, int my, cudaStream_t st) 
   return FFTBF_OK;
 }
 
-int tied_tc_launch(TiedTables& tt, const float* beams, int64_t nwin, int nfreq, int mx, int my,
-                   float* out, cudaStream_t st) {
-  const int64_t ntj = (nwin + ttc::TN - 1) / ttc::TN;
+template <int TN>
+static int tied_tc_run(TiedTables& tt, const float* beams, int64_t nwin, int nfreq, int mx, int my,
+                       float* out, cudaStream_t st) {
+  const int64_t ntj = (nwin + TN - 1) / TN;
   if (ntj > 65535 || nfreq > 65535)
     return set_error(FFTBF_EUNSUPPORTED, "tied beams: too many windows or channels per call");
-  const int64_t prow = (int64_t)nfreq * mx * ntj * ttc::TN;        // padded beam rows
+  const int64_t prow = (int64_t)nfreq * mx * ntj * TN;             // padded beam rows
   const int64_t erow = nwin * nfreq * mx;                           // exponents
   if ((size_t)prow > tt.p_cap) {
     cudaStreamSynchronize(st);                  // the old scratch may still be read
@@ -349,21 +410,28 @@ int tied_tc_launch(TiedTables& tt, const float* beams, int64_t nwin, int nfreq, 
     }
     tt.p_cap = (size_t)prow;
   }
-  const unsigned pblocks = (unsigned)std::min<int64_t>((prow + 7) / 8, 1 << 20);
-  tied_tc_prep_kernel<<<pblocks, 256, 0, st>>>(beams, nwin, nfreq, mx, my,
-                                               reinterpret_cast<__half*>(tt.ph),
-                                               reinterpret_cast<__half*>(tt.pl), tt.pe);
+  const unsigned pblocks = (unsigned)std::min<int64_t>((prow / 8 + 7) / 8, 1 << 20);
+  const int vec = (reinterpret_cast<uintptr_t>(beams) & 15) == 0;   // rows are multiples of 64 beams
+  tied_tc_prep_kernel<TN><<<pblocks, 256, 0, st>>>(beams, nwin, nfreq, mx, my,
+                                                   reinterpret_cast<__half*>(tt.ph),
+                                                   reinterpret_cast<__half*>(tt.pl), tt.pe, vec);
   FFTBF_CUDA_TRY(cudaGetLastError());
-  const size_t smem = ttc::NS * (size_t)ttc::STAGE;
-  FFTBF_CUDA_TRY(cudaFuncSetAttribute(tied_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  const size_t smem = ttc::Cfg<TN>::NS * (size_t)ttc::Cfg<TN>::STAGE;
+  FFTBF_CUDA_TRY(cudaFuncSetAttribute(tied_tc_kernel<TN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)smem));
   dim3 grid((tt.n_tied + ttc::TM - 1) / ttc::TM, (unsigned)ntj, nfreq);
-  tied_tc_kernel<<<grid, ttc::NT, smem, st>>>(
+  tied_tc_kernel<TN><<<grid, ttc::NT, smem, st>>>(
       reinterpret_cast<const __half*>(tt.wyh), reinterpret_cast<const __half*>(tt.wyl), tt.wye,
       tt.wa, tt.perm, reinterpret_cast<const __half*>(tt.ph), reinterpret_cast<const __half*>(tt.pl),
       tt.pe, out, nwin, nfreq, tt.n_tied, mx, my, tt.err);
   FFTBF_CUDA_TRY(cudaGetLastError());
   return FFTBF_OK;
+}
+
+int tied_tc_launch(TiedTables& tt, const float* beams, int64_t nwin, int nfreq, int mx, int my,
+                   float* out, cudaStream_t st) {
+  return nwin <= 64 ? tied_tc_run<64>(tt, beams, nwin, nfreq, mx, my, out, st)
+                    : tied_tc_run<128>(tt, beams, nwin, nfreq, mx, my, out, st);
 }
 
 }  // namespace fftbf

@@ -90,3 +90,29 @@ def test_tied_falls_back_to_cuda_cores_when_split_tables_do_not_fit(monkeypatch)
     monkeypatch.setenv("FFTBF_TIED_TC", "0")
     simt = _tied(P, shape, w, u, v, n_tied)
     assert np.array_equal(got, simt)                         # the same CUDA-core kernel ran
+
+
+@pytest.mark.parametrize("nwin", [1, 7, 63, 64, 65, 128])
+def test_tied_tensor_core_window_tiles_agree(nwin):
+    """Calls of at most 64 windows take 64-window tiles, larger ones 128-window tiles; every window
+    is the same product in both, so its beams are the same bits whichever call it is part of, and
+    also when the FFT beams start off a 16-byte boundary."""
+    nx, ny, mx, my, nfreq, n_tied = 4, 64, 4, 128, 3, 150
+    rng = np.random.default_rng(17)
+    P = rng.random((128, nfreq, mx, my), dtype=np.float32)
+    P[3] *= 2.0 ** -60                                       # rows scale by themselves
+    P[nwin - 1, 1] = 0.0
+    u = rng.integers(0, mx, (nfreq, n_tied)) / mx
+    v = rng.random((nfreq, n_tied))
+    def run(n, off):
+        buf = torch.empty(P[:n].size + 4, device="cuda")
+        P_dev = buf[off:off + P[:n].size].reshape(n, nfreq, mx, my)
+        P_dev.copy_(torch.from_numpy(P[:n]))
+        return _tied(P_dev, (nx, ny, mx, my, 1, nfreq, 8 * n, 8), None,
+                     u, v, n_tied)
+    got = run(nwin, 0)
+    scale = _scale(P[:nwin].astype(np.float64), u, v, nx, ny)
+    err = np.abs(got - oracle.tied_regrid(P[:nwin].astype(np.float64), u, v, nx, ny))
+    assert (err <= TOL_BEAM * scale).all()
+    assert np.array_equal(got, run(128, 0)[:nwin])
+    assert np.array_equal(got, run(nwin, 1))
