@@ -7,10 +7,10 @@
 // keeps FP32 accuracy; e scales every weight row and every beam row so that its largest
 // magnitude lies in [2^14, 2^15) (inside the FP16 range, with the residuals normal), and the
 // epilogue divides by 2^(e_s + e_j) exactly. Both split operands are stored in global
-// memory already cut into tiles (128 pointings or TN windows x 64 beams, the canonical K-major
+// memory already cut into tiles (128 pointings or TN windows x 32 beams, the canonical K-major
 // layout, zero rows past the ends). A CTA computes 128 pointings x TN windows of one channel: one
-// thread stages each K chunk as four bulk copies completing on a full-mbarrier (two or three
-// stages), issues its MMAs and commits them to the stage's empty-mbarrier; one TMEM
+// thread stages each K chunk as four bulk copies completing on a full-mbarrier (four or six
+// stages), another issues its MMAs and commits them to the stage's empty-mbarrier; one TMEM
 // accumulator of TN columns per E-W beam used by the tile's pointings, and each pointing
 // (TMEM lane) reads its own beam's accumulator. Every wait is bounded; a timeout sets the
 // plan's error word.
@@ -26,20 +26,21 @@
 namespace fftbf {
 
 namespace ttc {
-constexpr int TM = 128, KC = 64;               // pointings, beams per K chunk
-constexpr int LBO = 128, SBO = 1024;           // canonical K-major tile: 8 K blocks per row group
-constexpr int TILE = TM * KC * 2;              // bytes of one 128 x 64 FP16 tile
+constexpr int TM = 128, KC = 32;               // pointings, beams per K chunk
+constexpr int LBO = 128, SBO = 512;            // canonical K-major tile: 4 K blocks per row group
+constexpr int TILE = TM * KC * 2;              // bytes of one 128 x 32 FP16 tile
 constexpr int NT = 256;                        // warps w and w + 4 share TMEM lane quarter w % 4
 constexpr int MAXA = 4;                        // E-W beams (one accumulator each)
 // By windows per CTA TN: 128 in general; 64 for calls of at most 64 windows, where half of the MMA
 // columns and of the beam tiles would be padding, and where two CTAs then fit on an SM, so that
 // one's set-up and scattered stores run under the other's products. 256 channels x 2048 pointings
-// x 64 windows, whose split weights are 1.07 GB per call: 635 -> 415 us per call with the prep
-// kernel below.
+// x 64 windows, whose split weights are 1.07 GB per call (156 us at the copy rate): GEMM 516 us with
+// 128-window tiles, 336 with these, 245 with a copy thread of its own and chunks of 32 beams in
+// place of 64 (a stage is given back sooner, so more of the CTA's buffers are in flight).
 template <int TN> struct Cfg {
-  static constexpr int PT = TN * KC * 2;       // bytes of one TN x 64 beam tile
+  static constexpr int PT = TN * KC * 2;       // bytes of one TN x 32 beam tile
   static constexpr int STAGE = 2 * TILE + 2 * PT;   // W hi, W lo, P hi, P lo
-  static constexpr int NS = TN == 64 ? 2 : 3;  // staging buffers
+  static constexpr int NS = TN == 64 ? 4 : 6;  // staging buffers
   static constexpr int CTAS = TN == 64 ? 2 : 1;
   static constexpr uint32_t TMEM_COLS = MAXA * TN;
 };
@@ -49,11 +50,11 @@ constexpr uint64_t WAIT_NS = 1000000000ull;
 // e such that 2^e m lies in [2^14, 2^15) (0 for a zero row)
 __device__ __forceinline__ int split_exp(float m) { return m > 0.f ? 14 - ilogbf(m) : 0; }
 
-// Half offset of element (row r < 128, k) of a row tile: tile (k / 64) of the row tile's
+// Half offset of element (row r < 128, k) of a row tile: tile (k / 32) of the row tile's
 // chunks, canonical K-major layout inside.
 __device__ __forceinline__ int64_t tiled_off(int64_t tile0, int r, int k) {
-  return (tile0 + (k >> 6)) * (ttc::TILE / 2) +
-         (int64_t)(tc::kmajor_off(r, k & 63, ttc::LBO, ttc::SBO) >> 1);
+  return (tile0 + k / ttc::KC) * (ttc::TILE / 2) +
+         (int64_t)(tc::kmajor_off(r, k % ttc::KC, ttc::LBO, ttc::SBO) >> 1);
 }
 
 // Split one row x (one warp): hi and lo written at tiled_off(tile0, r, k), the row exponent
@@ -77,7 +78,7 @@ __device__ __forceinline__ int split_row_tiled(const float* x, float scale_in, i
 }
 
 // Weight tables in tiles: per channel, pointing tiles of 128 sorted slots (zero rows past
-// n_tied), each [my / 64] chunks of 128 x 64. Also the row's E-W beam A_s (the largest
+// n_tied), each [my / 32] chunks of 128 x 32. Also the row's E-W beam A_s (the largest
 // |wx|) and exponent; the row is wx[s, A_s] wy[s, :].
 __global__ void tied_tc_table_kernel(const float* __restrict__ wx, const float* __restrict__ wy,
                                      int nfreq, int n_tied, int mx, int my, __half* wyh,
@@ -115,66 +116,90 @@ __device__ __forceinline__ float scale_pow2(float x, int e) {
 }
 
 // Beam rows P[j, f, A, :] split the same way (per call), in tiles per (channel, E-W beam) of TN
-// windows (zero rows past nwin); exponents at pe[(j nfreq + f) mx + A]. A warp takes eight windows,
-// lane (g, r) eight beams of window r at a time: 128 contiguous bytes are read per window, and the
-// eight windows' 16-byte pieces of one K block are the 128 bytes of a core matrix, so every store
-// of the warp is 512 contiguous bytes (a row per warp wrote 16-byte pieces 128 bytes apart).
+// windows (zero rows past nwin); exponents at pe[(j nfreq + f) mx + A]. `wpg` warps take eight
+// windows: lane (g, r) holds eight beams of window r at a time, so 128 contiguous bytes are read
+// per window, and the eight windows' 16-byte pieces of one K block are the 128 bytes of a core
+// matrix: every store of a warp is 512 contiguous bytes (105 -> 59 us for 64 windows x 256 channels
+// x 4 x 512 beams, 134 MB read and 134 MB written, against a row per warp in 128-window tiles). A warp keeps its share of the rows in
+// registers between the row maximum and the split (up to kHold blocks of 32 beams; what is past
+// those is read again).
+constexpr int kPrepWarps = 8, kHold = 2;
 template <int TN>
-__global__ void tied_tc_prep_kernel(const float* __restrict__ P, int64_t nwin, int nfreq, int mx,
-                                    int my, __half* ph, __half* pl, int* pe, int vec) {
-  const int lane = threadIdx.x & 31, r = lane & 7, g = lane >> 3;
-  const int ntj = (int)((nwin + TN - 1) / TN), kcs = my / ttc::KC;
-  const int64_t per_fa = (int64_t)ntj * (TN / 8);      // groups of eight windows
-  const int64_t ngrp = (int64_t)nfreq * mx * per_fa;
-  const int64_t nw = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t gp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); gp < ngrp; gp += nw) {
-    const int64_t fa = gp / per_fa;                    // f mx + A
-    const int64_t j8 = gp - fa * per_fa, j = 8 * j8 + r;
-    const int f = (int)(fa / mx), A = (int)(fa - (int64_t)f * mx);
-    const bool live = j < nwin;
-    const float* x = P + ((live ? j * nfreq + f : 0) * mx + A) * my + 8 * g;
-    auto load = [&](int k, float (&v)[8]) {
-      if (vec) {
-        const float4 a = *reinterpret_cast<const float4*>(x + k), b = *reinterpret_cast<const float4*>(x + k + 4);
-        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-        v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-      } else {
+__global__ void __launch_bounds__(32 * kPrepWarps) tied_tc_prep_kernel(
+    const float* __restrict__ P, int64_t nwin, int nfreq, int mx, int my, __half* ph, __half* pl,
+    int* pe, int wpg, int vec) {
+  __shared__ float s_max[kPrepWarps][8];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = lane & 7, g = lane >> 3;
+  const int sub = warp % wpg, grp = warp / wpg;
+  const int ntj = (int)((nwin + TN - 1) / TN), nb = my / ttc::KC;
+  const int64_t per_fa = (int64_t)ntj * (TN / 8);        // groups of eight windows
+  const int64_t gp = (int64_t)blockIdx.x * (kPrepWarps / wpg) + grp;
+  const int64_t fa = gp / per_fa;                        // f mx + A
+  const int64_t j8 = gp - fa * per_fa, j = 8 * j8 + r;
+  const bool have = fa < (int64_t)nfreq * mx, live = have && j < nwin;
+  const int f = (int)(fa / mx), A = (int)(fa - (int64_t)f * mx);
+  const float* x = P + ((live ? j * nfreq + f : 0) * mx + (live ? A : 0)) * my + 8 * g;
+  auto load = [&](int b, float (&v)[8]) {                // beams 32 b + 8 g .. + 7
+    if (vec) {
+      const float4 a = *reinterpret_cast<const float4*>(x + 32 * b);
+      const float4 c = *reinterpret_cast<const float4*>(x + 32 * b + 4);
+      v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+      v[4] = c.x; v[5] = c.y; v[6] = c.z; v[7] = c.w;
+    } else {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] = x[k + i];
-      }
-    };
-    float m = 0.f;
-    if (live)
-#pragma unroll 4
-      for (int k = 0; k < my; k += 32) {
-        float v[8];
-        load(k, v);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) m = fmaxf(m, fabsf(v[i]));
-      }
-    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 8));
-    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
-    const int e = split_exp(m);
-    // this group's rows in the tile of chunk 0 (halves)
-    const int jt = (int)(8 * j8 / TN), row = (int)(8 * j8 - (int64_t)jt * TN);
-    const int64_t base = (fa * ntj + jt) * kcs * (TN * ttc::KC) + (row >> 3) * (ttc::SBO / 2) + lane * 8;
-#pragma unroll 4
-    for (int k = 0; k < my; k += 32) {
-      float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-      if (live) load(k, v);
-      __half2 h[4], l[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float a = scale_pow2(v[2 * i], e), b = scale_pow2(v[2 * i + 1], e);
-        h[i] = __halves2half2(__float2half_rn(a), __float2half_rn(b));
-        l[i] = __halves2half2(__float2half_rn(a - __low2float(h[i])), __float2half_rn(b - __high2float(h[i])));
-      }
-      const int64_t o = base + (int64_t)(k >> 6) * (TN * ttc::KC) + ((k & 63) >> 3) * (ttc::LBO / 2);
-      *reinterpret_cast<uint4*>(ph + o) = *reinterpret_cast<const uint4*>(h);
-      *reinterpret_cast<uint4*>(pl + o) = *reinterpret_cast<const uint4*>(l);
+      for (int i = 0; i < 8; ++i) v[i] = x[32 * b + i];
     }
-    if (live && g == 0) pe[(j * nfreq + f) * mx + A] = e;
+  };
+  float hold[kHold][8];
+  float m = 0.f;
+#pragma unroll
+  for (int q = 0; q < kHold; ++q) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) hold[q][i] = 0.f;
+    if (live && sub + q * wpg < nb) load(sub + q * wpg, hold[q]);
   }
+#pragma unroll
+  for (int q = 0; q < kHold; ++q)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) m = fmaxf(m, fabsf(hold[q][i]));
+  if (live)
+    for (int b = sub + kHold * wpg; b < nb; b += wpg) {
+      float v[8];
+      load(b, v);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) m = fmaxf(m, fabsf(v[i]));
+    }
+  m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 8));
+  m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
+  if (g == 0) s_max[warp][r] = m;
+  __syncthreads();
+  for (int w = 0; w < wpg; ++w) m = fmaxf(m, s_max[grp * wpg + w][r]);
+  if (!have) return;
+  const int e = split_exp(m);
+  // this group's rows in the tile of chunk 0 (halves)
+  const int jt = (int)(8 * j8 / TN), row = (int)(8 * j8 - (int64_t)jt * TN);
+  const int64_t base = (fa * ntj + jt) * nb * (TN * ttc::KC) + (row >> 3) * (ttc::SBO / 2) + lane * 8;
+  auto put = [&](int b, const float (&v)[8]) {
+    __half2 h[4], l[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float a = scale_pow2(v[2 * i], e), c = scale_pow2(v[2 * i + 1], e);
+      h[i] = __halves2half2(__float2half_rn(a), __float2half_rn(c));
+      l[i] = __halves2half2(__float2half_rn(a - __low2float(h[i])), __float2half_rn(c - __high2float(h[i])));
+    }
+    const int64_t o = base + (int64_t)b * (TN * ttc::KC);
+    *reinterpret_cast<uint4*>(ph + o) = *reinterpret_cast<const uint4*>(h);
+    *reinterpret_cast<uint4*>(pl + o) = *reinterpret_cast<const uint4*>(l);
+  };
+#pragma unroll
+  for (int q = 0; q < kHold; ++q)
+    if (sub + q * wpg < nb) put(sub + q * wpg, hold[q]);
+  for (int b = sub + kHold * wpg; b < nb; b += wpg) {
+    float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (live) load(b, v);
+    put(b, v);
+  }
+  if (live && g == 0 && sub == 0) pe[(j * nfreq + f) * mx + A] = e;
 }
 
 template <int TN>
@@ -188,7 +213,7 @@ __global__ void __launch_bounds__(ttc::NT, ttc::Cfg<TN>::CTAS) tied_tc_kernel(
   extern __shared__ __align__(1024) unsigned char smem_t[];
   __shared__ uint64_t full[NS], empty[NS];
   __shared__ uint32_t taddr;
-  __shared__ int s_mask;
+  __shared__ int s_mask, s_ok;
   __shared__ int s_pe[ttc::MAXA][TN];
   const int tid = threadIdx.x, warp = tid >> 5;
   const int f = blockIdx.z;
@@ -199,6 +224,9 @@ __global__ void __launch_bounds__(ttc::NT, ttc::Cfg<TN>::CTAS) tied_tc_kernel(
     tc::tmem_alloc(&taddr, C::TMEM_COLS);
     tc::tmem_relinquish();
   }
+  const int kcs = my / ttc::KC;
+  const int nts = (n_tied + ttc::TM - 1) / ttc::TM;
+  const int64_t wt0 = ((int64_t)f * nts + blockIdx.x) * kcs;   // first weight tile
   if (tid == 0) {
     for (int i = 0; i < NS; ++i) {
       tc::mbar_init(&full[i], 1);
@@ -206,15 +234,19 @@ __global__ void __launch_bounds__(ttc::NT, ttc::Cfg<TN>::CTAS) tied_tc_kernel(
     }
     tc::mbar_init_fence();
     s_mask = 0;
+    s_ok = 1;
   }
-  __syncthreads();
   const int row = tid & (ttc::TM - 1);           // TMEM lane / pointing of this thread
   const int s = s0 + row;
   const bool srow = s < n_tied;
   const int my_a = srow ? wa[fs0 + s] : 0;
   const int my_e = srow ? wye[fs0 + s] : 0;
-  if (srow && tid < ttc::TM) atomicOr(&s_mask, 1 << my_a);
+  const int dst_s = srow ? perm[fs0 + s] : 0;
   __syncthreads();
+  if (srow && tid < ttc::TM) atomicOr(&s_mask, 1 << my_a);
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
   const int mask = s_mask;
   int nact = 0, my_ai = 0;
   for (int A = 0; A < mx; ++A)
@@ -222,8 +254,8 @@ __global__ void __launch_bounds__(ttc::NT, ttc::Cfg<TN>::CTAS) tied_tc_kernel(
       if (A == my_a) my_ai = nact;
       ++nact;
     }
-  // exponents of the tile's windows, per E-W beam in use
-  for (int i = tid; i < nact * TN; i += ttc::NT) {
+  // exponents of the tile's windows, per E-W beam in use (warps 0 and 1 start on the pipeline)
+  for (int i = tid - 64; i >= 0 && i < nact * TN; i += ttc::NT - 64) {
     const int ai = i / TN, jj = i - ai * TN;
     int A = 0;
     for (int a = 0, c = -1; a < mx; ++a)
@@ -231,43 +263,40 @@ __global__ void __launch_bounds__(ttc::NT, ttc::Cfg<TN>::CTAS) tied_tc_kernel(
     const int64_t j = j0 + jj;
     s_pe[ai][jj] = j < nwin ? pe[(j * nfreq + f) * mx + A] : 0;
   }
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
   const uint32_t tbase = taddr;
-  const int kcs = my / ttc::KC;
   const int total = nact * kcs;
   const uint32_t idesc = tc::idesc_f16(ttc::TM, TN, false);
-  // Thread 0 runs the pipeline: chunk t = (E-W beam in use number t / kcs, K chunk t % kcs)
-  // goes to stage t % NS as four bulk copies completing on full[stage]; its MMAs
-  // commit to empty[stage], after which the stage takes chunk t + NS. The other threads wait
-  // at the CTA barrier. Every wait is bounded.
-  __shared__ int s_ok;
-  if (tid == 0) {
-    bool ok = true;
-    const int nts = (n_tied + ttc::TM - 1) / ttc::TM;
+  // Chunk t = (E-W beam in use number t / kcs, K chunk t % kcs) goes to stage t % NS. Thread 32
+  // stages the chunks as four bulk copies each, completing on full[stage]; thread 0 issues their
+  // MMAs and commits them to empty[stage], after which the stage takes chunk t + NS. One thread
+  // for both held each refill back until the next chunk's MMAs were issued. The other threads
+  // wait at the CTA barrier. Every wait is bounded.
+  if (tid == 32) {
     const int ntj = (int)((nwin + TN - 1) / TN);
-    const int64_t wt0 = ((int64_t)f * nts + blockIdx.x) * kcs;   // first weight tile
-    auto issue = [&](int t) {
-      const int st = t % NS;
-      unsigned char* stg = smem_t + st * STAGE;
-      const int ai = t / kcs, kc = t - ai * kcs;
-      int A = 0;
-      for (int a = 0, c = -1; a < mx; ++a)
-        if ((mask >> a) & 1 && ++c == ai) A = a;
-      const int64_t pt = (((int64_t)f * mx + A) * ntj + blockIdx.y) * kcs + kc;
-      const int64_t wt = wt0 + kc;
-      tc::mbar_arrive_expect_tx(&full[st], (uint32_t)STAGE);
-      tc::bulk_g2s(stg, wyh + wt * (ttc::TILE / 2), ttc::TILE, &full[st]);
-      tc::bulk_g2s(stg + ttc::TILE, wyl + wt * (ttc::TILE / 2), ttc::TILE, &full[st]);
-      tc::bulk_g2s(stg + 2 * ttc::TILE, ph + pt * (PT / 2), PT, &full[st]);
-      tc::bulk_g2s(stg + 2 * ttc::TILE + PT, pl + pt * (PT / 2), PT, &full[st]);
-    };
-    for (int t = 0; t < NS && t < total; ++t) issue(t);
+    bool ok = true;
+    int t = 0;
+    for (int A = 0; A < mx && ok; ++A) {
+      if (!((mask >> A) & 1)) continue;
+      const int64_t pt0 = (((int64_t)f * mx + A) * ntj + blockIdx.y) * kcs;
+      for (int kc = 0; kc < kcs; ++kc, ++t) {
+        const int st = t % NS;
+        if (t >= NS) ok = tc::mbar_wait(&empty[st], (uint32_t)((t / NS - 1) & 1), ttc::WAIT_NS);
+        if (!ok) break;
+        unsigned char* stg = smem_t + st * STAGE;
+        const int64_t wt = (wt0 + kc) * (ttc::TILE / 2), pt = (pt0 + kc) * (PT / 2);
+        tc::mbar_arrive_expect_tx(&full[st], (uint32_t)STAGE);
+        tc::bulk_g2s(stg, wyh + wt, ttc::TILE, &full[st]);
+        tc::bulk_g2s(stg + ttc::TILE, wyl + wt, ttc::TILE, &full[st]);
+        tc::bulk_g2s(stg + 2 * ttc::TILE, ph + pt, PT, &full[st]);
+        tc::bulk_g2s(stg + 2 * ttc::TILE + PT, pl + pt, PT, &full[st]);
+      }
+    }
+    if (!ok) atomicExch(&s_ok, 0);
+  } else if (tid == 0) {
+    bool ok = true;
     for (int t = 0; t < total && ok; ++t) {
       const int st = t % NS;
-      const uint32_t par = (uint32_t)((t / NS) & 1);
-      ok = tc::mbar_wait(&full[st], par, ttc::WAIT_NS);
+      ok = tc::mbar_wait(&full[st], (uint32_t)((t / NS) & 1), ttc::WAIT_NS);
       if (!ok) break;
       tc::fence_after_sync();
       const uint32_t sa = tc::smem_u32(smem_t + st * STAGE);
@@ -285,18 +314,12 @@ __global__ void __launch_bounds__(ttc::NT, ttc::Cfg<TN>::CTAS) tied_tc_kernel(
         tc::mma_f16(d, dwl, dph, idesc, 1u);
       }
       tc::mma_commit(&empty[st]);
-      // refill the stage of chunk t - 1 once its MMAs are done
-      const int tp = t - 1;
-      if (tp >= 0 && tp + NS < total) {
-        ok = tc::mbar_wait(&empty[tp % NS], (uint32_t)((tp / NS) & 1), ttc::WAIT_NS);
-        if (ok) issue(tp + NS);
-      }
     }
     if (ok && total > 0) {                          // the last commit covers every MMA
       const int tl = total - 1;
       ok = tc::mbar_wait(&empty[tl % NS], (uint32_t)((tl / NS) & 1), ttc::WAIT_NS);
     }
-    s_ok = ok ? 1 : 0;
+    if (!ok) atomicExch(&s_ok, 0);
   }
   tc::fence_before_sync();
   __syncthreads();
@@ -305,7 +328,6 @@ __global__ void __launch_bounds__(ttc::NT, ttc::Cfg<TN>::CTAS) tied_tc_kernel(
   if (ok && total > 0) {
     // warp w reads TMEM lanes 32 (w % 4) .. + 31 (its pointings) and half w / 4 of the windows
     const uint32_t lane_off = (uint32_t)(32 * (warp & 3)) << 16;
-    const int dst_s = srow ? perm[fs0 + s] : 0;
     for (int c = TN / 64 * (warp >> 2); c < TN / 64 * (warp >> 2) + TN / 64; ++c) {
       for (int a2 = 0; a2 < nact; ++a2) {
         uint32_t r[32];
@@ -338,7 +360,7 @@ __global__ void __launch_bounds__(ttc::NT, ttc::Cfg<TN>::CTAS) tied_tc_kernel(
 bool tied_tc_eligible(bool dense_x, int mx, int my) {
   const char* env = getenv("FFTBF_TIED_TC");
   if (env && env[0] == '0') return false;
-  return !dense_x && mx <= ttc::MAXA && my >= ttc::KC && my % ttc::KC == 0;
+  return !dense_x && mx <= ttc::MAXA && my >= 64 && my % 64 == 0;
 }
 
 int tied_tc_build(TiedTables& tt, int64_t nuv, int mx, int my, cudaStream_t st) {
@@ -387,8 +409,10 @@ static int tied_tc_run(TiedTables& tt, const float* beams, int64_t nwin, int nfr
   if (ntj > 65535 || nfreq > 65535)
     return set_error(FFTBF_EUNSUPPORTED, "tied beams: too many windows or channels per call");
   const int64_t prow = (int64_t)nfreq * mx * ntj * TN;             // padded beam rows
+  // scratch rows: to whole 128 windows, so that calls on either side of the rule share it
+  const int64_t crow = (int64_t)nfreq * mx * ((nwin + 127) / 128) * 128;
   const int64_t erow = nwin * nfreq * mx;                           // exponents
-  if ((size_t)prow > tt.p_cap) {
+  if ((size_t)crow > tt.p_cap) {
     cudaStreamSynchronize(st);                  // the old scratch may still be read
     cudaFree(tt.ph);
     cudaFree(tt.pl);
@@ -396,9 +420,9 @@ static int tied_tc_run(TiedTables& tt, const float* beams, int64_t nwin, int nfr
     tt.ph = tt.pl = nullptr;
     tt.pe = nullptr;
     tt.p_cap = 0;
-    bool ok = cudaMalloc(&tt.ph, prow * my * sizeof(__half)) == cudaSuccess &&
-              cudaMalloc(&tt.pl, prow * my * sizeof(__half)) == cudaSuccess &&
-              cudaMalloc(&tt.pe, std::max<int64_t>(erow, prow) * sizeof(int)) == cudaSuccess;
+    bool ok = cudaMalloc(&tt.ph, crow * my * sizeof(__half)) == cudaSuccess &&
+              cudaMalloc(&tt.pl, crow * my * sizeof(__half)) == cudaSuccess &&
+              cudaMalloc(&tt.pe, std::max<int64_t>(erow, crow) * sizeof(int)) == cudaSuccess;
     if (!ok) {
       cudaGetLastError();
       cudaFree(tt.ph);
@@ -408,13 +432,16 @@ static int tied_tc_run(TiedTables& tt, const float* beams, int64_t nwin, int nfr
       tt.pe = nullptr;
       return set_error(FFTBF_ENOMEM, "cannot allocate the split beam scratch");
     }
-    tt.p_cap = (size_t)prow;
+    tt.p_cap = (size_t)crow;
   }
-  const unsigned pblocks = (unsigned)std::min<int64_t>((prow / 8 + 7) / 8, 1 << 20);
+  // two blocks of 32 beams per warp where the row is long enough, so that a warp's loads are all
+  // in flight at once and a short call still has many warps
+  const int wpg = my >= 512 ? 8 : my >= 256 ? 4 : my >= 128 ? 2 : 1;
+  const int64_t gpb = kPrepWarps / wpg, pblocks = (prow / 8 + gpb - 1) / gpb;
   const int vec = (reinterpret_cast<uintptr_t>(beams) & 15) == 0;   // rows are multiples of 64 beams
-  tied_tc_prep_kernel<TN><<<pblocks, 256, 0, st>>>(beams, nwin, nfreq, mx, my,
-                                                   reinterpret_cast<__half*>(tt.ph),
-                                                   reinterpret_cast<__half*>(tt.pl), tt.pe, vec);
+  tied_tc_prep_kernel<TN><<<(unsigned)pblocks, 32 * kPrepWarps, 0, st>>>(
+      beams, nwin, nfreq, mx, my, reinterpret_cast<__half*>(tt.ph),
+      reinterpret_cast<__half*>(tt.pl), tt.pe, wpg, vec);
   FFTBF_CUDA_TRY(cudaGetLastError());
   const size_t smem = ttc::Cfg<TN>::NS * (size_t)ttc::Cfg<TN>::STAGE;
   FFTBF_CUDA_TRY(cudaFuncSetAttribute(tied_tc_kernel<TN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
