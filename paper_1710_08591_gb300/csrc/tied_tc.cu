@@ -7,12 +7,12 @@
 // keeps FP32 accuracy; e scales every weight row and every beam row so that its largest
 // magnitude lies in [2^14, 2^15) (inside the FP16 range, with the residuals normal), and the
 // epilogue divides by 2^(e_s + e_j) exactly. Both split operands are stored in global
-// memory already cut into tiles (128 pointings or TN windows x 32 beams, the canonical K-major
-// layout, zero rows past the ends). A CTA computes 128 pointings x TN windows of one channel: one
-// thread stages each K chunk as four bulk copies completing on a full-mbarrier (four or six
-// stages), another issues its MMAs and commits them to the stage's empty-mbarrier; one TMEM
-// accumulator of TN columns per E-W beam used by the tile's pointings, and each pointing
-// (TMEM lane) reads its own beam's accumulator. Every wait is bounded; a timeout sets the
+// memory already cut into tiles (128 pointings or 64 windows x 32 beams, the canonical K-major
+// layout, zero rows past the ends). A CTA computes 128 pointings x 64 windows of one channel: one
+// thread stages each K chunk as four bulk copies completing on a full-mbarrier (four stages),
+// another issues its MMAs and commits them to the stage's empty-mbarrier; one TMEM accumulator
+// of 64 columns per E-W beam used by the tile's pointings, and each pointing (TMEM lane) reads
+// its own beam's accumulator. Every wait is bounded; a timeout sets the
 // plan's error word.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -31,19 +31,18 @@ constexpr int LBO = 128, SBO = 512;            // canonical K-major tile: 4 K bl
 constexpr int TILE = TM * KC * 2;              // bytes of one 128 x 32 FP16 tile
 constexpr int NT = 256;                        // warps w and w + 4 share TMEM lane quarter w % 4
 constexpr int MAXA = 4;                        // E-W beams (one accumulator each)
-// By windows per CTA TN: 128 in general; 64 for calls of at most 64 windows, where half of the MMA
-// columns and of the beam tiles would be padding, and where two CTAs then fit on an SM, so that
-// one's set-up and scattered stores run under the other's products. 256 channels x 2048 pointings
-// x 64 windows, whose split weights are 1.07 GB per call (156 us at the copy rate): GEMM 516 us with
-// 128-window tiles, 336 with these, 245 with a copy thread of its own and chunks of 32 beams in
-// place of 64 (a stage is given back sooner, so more of the CTA's buffers are in flight).
-template <int TN> struct Cfg {
-  static constexpr int PT = TN * KC * 2;       // bytes of one TN x 32 beam tile
-  static constexpr int STAGE = 2 * TILE + 2 * PT;   // W hi, W lo, P hi, P lo
-  static constexpr int NS = TN == 64 ? 4 : 6;  // staging buffers
-  static constexpr int CTAS = TN == 64 ? 2 : 1;
-  static constexpr uint32_t TMEM_COLS = MAXA * TN;
-};
+// Windows per CTA. 64, because two CTAs then fit on an SM, so that one's set-up and scattered stores
+// run under the other's products; the second window tile of a channel finds the weights in L2.
+// 256 channels x 2048 pointings, whose split weights are 1.07 GB per call (156 us at the copy rate),
+// against tiles of 128 windows with one CTA per SM: 245 for 482 us at 64 windows, 416 for 482 at 128,
+// 783 for 921 at 256; 64 channels x 300 pointings x 128 windows of 4x64: 21 for 28 us.
+constexpr int TN = 64;
+constexpr int PT = TN * KC * 2;                // bytes of one TN x 32 beam tile
+constexpr int STAGE = 2 * TILE + 2 * PT;       // W hi, W lo, P hi, P lo
+// Staging buffers. Chunks of 32 beams in four rather than of 64 in two: a stage is given back sooner,
+// so more of the buffers are in flight (336 -> 245 us at 64 windows, with the copy thread).
+constexpr int NS = 4;
+constexpr uint32_t TMEM_COLS = MAXA * TN;
 constexpr uint64_t WAIT_NS = 1000000000ull;
 }  // namespace ttc
 
@@ -115,22 +114,23 @@ __device__ __forceinline__ float scale_pow2(float x, int e) {
   return e >= -126 && e <= 127 ? x * __int_as_float((127 + e) << 23) : ldexpf(x, e);
 }
 
-// Beam rows P[j, f, A, :] split the same way (per call), in tiles per (channel, E-W beam) of TN
+// Beam rows P[j, f, A, :] split the same way (per call), in tiles per (channel, E-W beam) of 64
 // windows (zero rows past nwin); exponents at pe[(j nfreq + f) mx + A]. `wpg` warps take eight
 // windows: lane (g, r) holds eight beams of window r at a time, so 128 contiguous bytes are read
 // per window, and the eight windows' 16-byte pieces of one K block are the 128 bytes of a core
-// matrix: every store of a warp is 512 contiguous bytes (105 -> 59 us for 64 windows x 256 channels
-// x 4 x 512 beams, 134 MB read and 134 MB written, against a row per warp in 128-window tiles). A warp keeps its share of the rows in
+// matrix: every store of a warp is 512 contiguous bytes. A warp keeps its share of the rows in
 // registers between the row maximum and the split (up to kHold blocks of 32 beams; what is past
-// those is read again).
+// those is read again). Bound by memory: 134 MB read and 134 MB written for 64 windows x 256
+// channels x 4 x 512 beams in 59 us (4.6 TB/s); with the rows read
+// twice instead it took 80 us.
 constexpr int kPrepWarps = 8, kHold = 2;
-template <int TN>
 __global__ void __launch_bounds__(32 * kPrepWarps) tied_tc_prep_kernel(
     const float* __restrict__ P, int64_t nwin, int nfreq, int mx, int my, __half* ph, __half* pl,
     int* pe, int wpg, int vec) {
   __shared__ float s_max[kPrepWarps][8];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = lane & 7, g = lane >> 3;
   const int sub = warp % wpg, grp = warp / wpg;
+  using ttc::TN;
   const int ntj = (int)((nwin + TN - 1) / TN), nb = my / ttc::KC;
   const int64_t per_fa = (int64_t)ntj * (TN / 8);        // groups of eight windows
   const int64_t gp = (int64_t)blockIdx.x * (kPrepWarps / wpg) + grp;
@@ -202,14 +202,12 @@ __global__ void __launch_bounds__(32 * kPrepWarps) tied_tc_prep_kernel(
   if (live && g == 0 && sub == 0) pe[(j * nfreq + f) * mx + A] = e;
 }
 
-template <int TN>
-__global__ void __launch_bounds__(ttc::NT, ttc::Cfg<TN>::CTAS) tied_tc_kernel(
+__global__ void __launch_bounds__(ttc::NT, 2) tied_tc_kernel(
     const __half* __restrict__ wyh, const __half* __restrict__ wyl, const int* __restrict__ wye,
     const int* __restrict__ wa, const int* __restrict__ perm, const __half* __restrict__ ph,
     const __half* __restrict__ pl, const int* __restrict__ pe, float* __restrict__ out,
     int64_t nwin, int nfreq, int n_tied, int mx, int my, int* err) {
-  using C = ttc::Cfg<TN>;
-  constexpr int NS = C::NS, STAGE = C::STAGE, PT = C::PT;
+  using ttc::NS, ttc::PT, ttc::STAGE, ttc::TN;
   extern __shared__ __align__(1024) unsigned char smem_t[];
   __shared__ uint64_t full[NS], empty[NS];
   __shared__ uint32_t taddr;
@@ -217,16 +215,18 @@ __global__ void __launch_bounds__(ttc::NT, ttc::Cfg<TN>::CTAS) tied_tc_kernel(
   __shared__ int s_pe[ttc::MAXA][TN];
   const int tid = threadIdx.x, warp = tid >> 5;
   const int f = blockIdx.z;
-  const int s0 = blockIdx.x * ttc::TM;
-  const int64_t j0 = (int64_t)blockIdx.y * TN;
+  // pointing tiles run fastest, window tiles next, channels last
+  const int nts = (n_tied + ttc::TM - 1) / ttc::TM;
+  const int jt = (int)(blockIdx.x / (unsigned)nts), pt_i = (int)(blockIdx.x - (unsigned)jt * nts);
+  const int s0 = pt_i * ttc::TM;
+  const int64_t j0 = (int64_t)jt * TN;
   const int64_t fs0 = (int64_t)f * n_tied;
   if (warp == 0) {
-    tc::tmem_alloc(&taddr, C::TMEM_COLS);
+    tc::tmem_alloc(&taddr, ttc::TMEM_COLS);
     tc::tmem_relinquish();
   }
   const int kcs = my / ttc::KC;
-  const int nts = (n_tied + ttc::TM - 1) / ttc::TM;
-  const int64_t wt0 = ((int64_t)f * nts + blockIdx.x) * kcs;   // first weight tile
+  const int64_t wt0 = ((int64_t)f * nts + pt_i) * kcs;   // first weight tile
   if (tid == 0) {
     for (int i = 0; i < NS; ++i) {
       tc::mbar_init(&full[i], 1);
@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(ttc::NT, ttc::Cfg<TN>::CTAS) tied_tc_kernel(
     int t = 0;
     for (int A = 0; A < mx && ok; ++A) {
       if (!((mask >> A) & 1)) continue;
-      const int64_t pt0 = (((int64_t)f * mx + A) * ntj + blockIdx.y) * kcs;
+      const int64_t pt0 = (((int64_t)f * mx + A) * ntj + jt) * kcs;
       for (int kc = 0; kc < kcs; ++kc, ++t) {
         const int st = t % NS;
         if (t >= NS) ok = tc::mbar_wait(&empty[st], (uint32_t)((t / NS - 1) & 1), ttc::WAIT_NS);
@@ -328,22 +328,21 @@ __global__ void __launch_bounds__(ttc::NT, ttc::Cfg<TN>::CTAS) tied_tc_kernel(
   if (ok && total > 0) {
     // warp w reads TMEM lanes 32 (w % 4) .. + 31 (its pointings) and half w / 4 of the windows
     const uint32_t lane_off = (uint32_t)(32 * (warp & 3)) << 16;
-    for (int c = TN / 64 * (warp >> 2); c < TN / 64 * (warp >> 2) + TN / 64; ++c) {
-      for (int a2 = 0; a2 < nact; ++a2) {
-        uint32_t r[32];
-        tc::tmem_ld32(tbase + lane_off + (uint32_t)(a2 * TN + 32 * c), r);
-        tc::tmem_wait_ld();
-        if (a2 == my_ai && srow) {
+    const int c = warp >> 2;
+    for (int a2 = 0; a2 < nact; ++a2) {
+      uint32_t r[32];
+      tc::tmem_ld32(tbase + lane_off + (uint32_t)(a2 * TN + 32 * c), r);
+      tc::tmem_wait_ld();
+      if (a2 == my_ai && srow) {
 #pragma unroll
-          for (int q = 0; q < 32; ++q) {
-            const int64_t j = j0 + 32 * c + q;
-            if (j < nwin) {
-              // D 2^-E: a power-of-two product (exact) while 2^-E is a normal float
-              const int E = my_e + s_pe[a2][32 * c + q];
-              const float d = __uint_as_float(r[q]);
-              out[(j * nfreq + f) * (int64_t)n_tied + dst_s] =
-                  (E > -127 && E < 127) ? d * __int_as_float((127 - E) << 23) : ldexpf(d, -E);
-            }
+        for (int q = 0; q < 32; ++q) {
+          const int64_t j = j0 + 32 * c + q;
+          if (j < nwin) {
+            // D 2^-E: a power-of-two product (exact) while 2^-E is a normal float
+            const int E = my_e + s_pe[a2][32 * c + q];
+            const float d = __uint_as_float(r[q]);
+            out[(j * nfreq + f) * (int64_t)n_tied + dst_s] =
+                (E > -127 && E < 127) ? d * __int_as_float((127 - E) << 23) : ldexpf(d, -E);
           }
         }
       }
@@ -353,7 +352,7 @@ __global__ void __launch_bounds__(ttc::NT, ttc::Cfg<TN>::CTAS) tied_tc_kernel(
   }
   tc::fence_before_sync();
   __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tbase, C::TMEM_COLS);
+  if (warp == 0) tc::tmem_dealloc(tbase, ttc::TMEM_COLS);
 }
 
 // ------------------------------------------------------------------------------ host --
@@ -402,16 +401,17 @@ int tied_tc_build(TiedTables& tt, int64_t nuv, int mx, int my, cudaStream_t st) 
   return FFTBF_OK;
 }
 
-template <int TN>
-static int tied_tc_run(TiedTables& tt, const float* beams, int64_t nwin, int nfreq, int mx, int my,
-                       float* out, cudaStream_t st) {
+int tied_tc_launch(TiedTables& tt, const float* beams, int64_t nwin, int nfreq, int mx, int my,
+                   float* out, cudaStream_t st) {
+  using ttc::TN;
   const int64_t ntj = (nwin + TN - 1) / TN;
-  if (ntj > 65535 || nfreq > 65535)
+  const int64_t nts = (tt.n_tied + ttc::TM - 1) / ttc::TM;
+  if ((nwin + 127) / 128 > 65535 || nfreq > 65535 || nts * ntj > INT32_MAX)
     return set_error(FFTBF_EUNSUPPORTED, "tied beams: too many windows or channels per call");
   const int64_t prow = (int64_t)nfreq * mx * ntj * TN;             // padded beam rows
-  // scratch rows: to whole 128 windows, so that calls on either side of the rule share it
+  // scratch rows and exponents for the next whole 128 windows: a call of a few more windows than
+  // an earlier one, possibly under capture, then seldom has to allocate
   const int64_t crow = (int64_t)nfreq * mx * ((nwin + 127) / 128) * 128;
-  const int64_t erow = nwin * nfreq * mx;                           // exponents
   if ((size_t)crow > tt.p_cap) {
     cudaStreamSynchronize(st);                  // the old scratch may still be read
     cudaFree(tt.ph);
@@ -422,7 +422,7 @@ static int tied_tc_run(TiedTables& tt, const float* beams, int64_t nwin, int nfr
     tt.p_cap = 0;
     bool ok = cudaMalloc(&tt.ph, crow * my * sizeof(__half)) == cudaSuccess &&
               cudaMalloc(&tt.pl, crow * my * sizeof(__half)) == cudaSuccess &&
-              cudaMalloc(&tt.pe, std::max<int64_t>(erow, crow) * sizeof(int)) == cudaSuccess;
+              cudaMalloc(&tt.pe, crow * sizeof(int)) == cudaSuccess;
     if (!ok) {
       cudaGetLastError();
       cudaFree(tt.ph);
@@ -439,26 +439,20 @@ static int tied_tc_run(TiedTables& tt, const float* beams, int64_t nwin, int nfr
   const int wpg = my >= 512 ? 8 : my >= 256 ? 4 : my >= 128 ? 2 : 1;
   const int64_t gpb = kPrepWarps / wpg, pblocks = (prow / 8 + gpb - 1) / gpb;
   const int vec = (reinterpret_cast<uintptr_t>(beams) & 15) == 0;   // rows are multiples of 64 beams
-  tied_tc_prep_kernel<TN><<<(unsigned)pblocks, 32 * kPrepWarps, 0, st>>>(
+  tied_tc_prep_kernel<<<(unsigned)pblocks, 32 * kPrepWarps, 0, st>>>(
       beams, nwin, nfreq, mx, my, reinterpret_cast<__half*>(tt.ph),
       reinterpret_cast<__half*>(tt.pl), tt.pe, wpg, vec);
   FFTBF_CUDA_TRY(cudaGetLastError());
-  const size_t smem = ttc::Cfg<TN>::NS * (size_t)ttc::Cfg<TN>::STAGE;
-  FFTBF_CUDA_TRY(cudaFuncSetAttribute(tied_tc_kernel<TN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  const size_t smem = ttc::NS * (size_t)ttc::STAGE;
+  FFTBF_CUDA_TRY(cudaFuncSetAttribute(tied_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)smem));
-  dim3 grid((tt.n_tied + ttc::TM - 1) / ttc::TM, (unsigned)ntj, nfreq);
-  tied_tc_kernel<TN><<<grid, ttc::NT, smem, st>>>(
+  dim3 grid((unsigned)(nts * ntj), 1, nfreq);
+  tied_tc_kernel<<<grid, ttc::NT, smem, st>>>(
       reinterpret_cast<const __half*>(tt.wyh), reinterpret_cast<const __half*>(tt.wyl), tt.wye,
       tt.wa, tt.perm, reinterpret_cast<const __half*>(tt.ph), reinterpret_cast<const __half*>(tt.pl),
       tt.pe, out, nwin, nfreq, tt.n_tied, mx, my, tt.err);
   FFTBF_CUDA_TRY(cudaGetLastError());
   return FFTBF_OK;
-}
-
-int tied_tc_launch(TiedTables& tt, const float* beams, int64_t nwin, int nfreq, int mx, int my,
-                   float* out, cudaStream_t st) {
-  return nwin <= 64 ? tied_tc_run<64>(tt, beams, nwin, nfreq, mx, my, out, st)
-                    : tied_tc_run<128>(tt, beams, nwin, nfreq, mx, my, out, st);
 }
 
 }  // namespace fftbf

@@ -94,9 +94,8 @@ def test_tied_falls_back_to_cuda_cores_when_split_tables_do_not_fit(monkeypatch)
 
 @pytest.mark.parametrize("nwin", [1, 7, 63, 64, 65, 128])
 def test_tied_tensor_core_window_tiles_agree(nwin):
-    """Calls of at most 64 windows take 64-window tiles, larger ones 128-window tiles; every window
-    is the same product in both, so its beams are the same bits whichever call it is part of, and
-    also when the FFT beams start off a 16-byte boundary."""
+    """Tiles of 64 windows, full and partial, one and two: every window's beams are the same bits
+    whichever call it is part of, and also when the FFT beams start off a 16-byte boundary."""
     nx, ny, mx, my, nfreq, n_tied = 4, 64, 4, 128, 3, 150
     rng = np.random.default_rng(17)
     P = rng.random((128, nfreq, mx, my), dtype=np.float32)
