@@ -14,7 +14,15 @@
 // (2n - 1) e mod 2 = [((2n - 1)(ih - B) mod 2M) + (2n - 1) fr] / M are formed from exact
 // integers plus one FP32 term; the weights w = sin((2n-1) pi e) / (M sin(pi e)) and their
 // derivative then come from FP32 sinpi/cospi, with a series near e = 0. The final sum of
-// the pointed beam is accumulated in FP64.
+// the pointed beam is a compensated FP32 sum; there both sines of a beam away from the estimate
+// come from the angle addition of a table at the integer part and the estimate's fraction.
+//
+// Bound by instruction issue and by the chain of each Newton step, not by the one reading of the
+// beams (268 MB for 32768 items of 4x512, 39 us at the copy rate). 5 steps of 10 taps there: 147 us
+// with every sine computed, a compare and two selects per beam in the search for the maximum and four
+// CTAs per SM (3870 warp instructions per item); 132 us with the table, the search by four beams and
+// the two sines of a tap in two lanes; 118 us at five CTAs per SM (48 registers, no spills; six
+// spill). 8192 items of 8x128: 24 us.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -26,6 +34,10 @@ namespace fftbf {
 
 constexpr int kLocTaps = 64;          // most taps per axis
 constexpr int kLocWarps = 8;
+// Largest M whose (sin, cos)(pi k / M), k < 2M, are kept in shared memory for the final sum over the
+// beams of the second axis: 32 KB, so that five CTAs stay resident. Below 32 beams most lie within
+// the eight of the direct sines and the table would cost as much as it saves.
+constexpr int kLocTab = 2048;
 
 struct LocAxis {
   int n, M, fit;
@@ -40,22 +52,32 @@ __device__ __forceinline__ int mod_m(const LocAxis& ax, int k) {
   return r < 0 ? r + ax.M : r;
 }
 
-// Dirichlet regridding weight of FFT beam B at the position (ih, fr), and its y-derivative.
-__device__ __forceinline__ void dir_weight(const LocAxis& ax, int ih, float fr, int B, float* w,
-                                           float* dw) {
-  const int M = ax.M, L = 2 * ax.n - 1;
+// The angles of FFT beam B at the position (ih, fr): e = y - B/M reduced to [-1/2, 1/2), its integer
+// part d in beams, the phase (2n - 1) e mod 2 (ph) and that of d (m2, any representative mod 2M).
+__device__ __forceinline__ void dir_d(const LocAxis& ax, int ih, float fr, int B, int* d_, float* r) {
   int d = mod_m(ax, ih - B);                          // e M = d + fr, reduced to [-M/2, M/2)
-  if ((float)d + fr >= 0.5f * M) d -= M;
-  const float r = (float)d + fr;
-  const float e = r * ax.invM;
+  if ((float)d + fr >= 0.5f * ax.M) d -= ax.M;
+  *d_ = d;
+  *r = (float)d + fr;
+}
+__device__ __forceinline__ int dir_m2(const LocAxis& ax, int d) {
+  const int M = ax.M, L = 2 * ax.n - 1;
   // (2n - 1) d mod 2M, any representative: |L d| <= M^2 / 2 + M fits 32 bits for M <= 32768
-  const int m2 = ax.pow2 ? ((L * d) & (2 * M - 1))
-                         : (M <= 32768 ? (L * d) % (2 * M) : (int)(((long long)L * d) % (2LL * M)));
-  float ph = ((float)m2 + (float)L * fr) * ax.invM;   // (2n - 1) e  (mod 2)
-  ph -= 2.f * rintf(0.5f * ph);
-  float sL, cL, s1, c1;
-  sincospif(ph, &sL, &cL);
-  sincospif(e, &s1, &c1);
+  return ax.pow2 ? ((L * d) & (2 * M - 1))
+                 : (M <= 32768 ? (L * d) % (2 * M) : (int)(((long long)L * d) % (2LL * M)));
+}
+__device__ __forceinline__ void dir_angles(const LocAxis& ax, int ih, float fr, int B, float* e, float* ph) {
+  int d;
+  float r;
+  dir_d(ax, ih, fr, B, &d, &r);
+  *e = r * ax.invM;
+  const float L = (float)(2 * ax.n - 1);
+  const float p = ((float)dir_m2(ax, d) + L * fr) * ax.invM;   // (2n - 1) e  (mod 2)
+  *ph = p - 2.f * rintf(0.5f * p);
+}
+__device__ __forceinline__ void dir_value(const LocAxis& ax, float e, float sL, float cL, float s1,
+                                          float c1, float* w, float* dw) {
+  const int M = ax.M, L = 2 * ax.n - 1;
   const float Le = (float)L * e;
   if (fabsf(Le) < 0.05f) {
     // f(x) = sin(Lx)/sin(x) = L[1 + x^2 (1 - L^2)/6 + x^4 (7/360 - L^2/36 + L^4/120)] + ...
@@ -68,6 +90,35 @@ __device__ __forceinline__ void dir_weight(const LocAxis& ax, int ih, float fr, 
     *w = sL / (s1 * (float)M);
     *dw = 3.14159265358979f * ax.invM * ((float)L * cL * s1 - sL * c1) / (s1 * s1);
   }
+}
+
+// Dirichlet regridding weight of FFT beam B at the position (ih, fr), and its y-derivative.
+__device__ __forceinline__ void dir_weight(const LocAxis& ax, int ih, float fr, int B, float* w,
+                                           float* dw) {
+  float e, ph, sL, cL, s1, c1;
+  dir_angles(ax, ih, fr, B, &e, &ph);
+  sincospif(ph, &sL, &cL);
+  sincospif(e, &s1, &c1);
+  dir_value(ax, e, sL, cL, s1, c1, w, dw);
+}
+// The same by a warp for up to 16 beams: lanes t and t + 16 (both given lane t's beam) take one
+// sine and cosine each. The results are lanes 0 - 15's.
+__device__ __forceinline__ void dir_weight_pair(const LocAxis& ax, int ih, float fr, int B, int lane,
+                                                float* w, float* dw) {
+  float e, ph, s, c;
+  dir_angles(ax, ih, fr, B, &e, &ph);
+  sincospif(lane < 16 ? ph : e, &s, &c);
+  const float s1 = __shfl_xor_sync(0xffffffffu, s, 16), c1 = __shfl_xor_sync(0xffffffffu, c, 16);
+  dir_value(ax, e, s, c, s1, c1, w, dw);
+}
+
+// (sin, cos)(pi x / M), x = a * fr, with the rounding errors of a fr and of the quotient put back.
+__device__ __forceinline__ float2 frac_angle(const LocAxis& ax, float a, float fr) {
+  const float p = a * fr, q = p * ax.invM;
+  const float lo = 3.14159265358979f * ((fmaf(-q, (float)ax.M, p) + fmaf(a, fr, -p)) * ax.invM);
+  float s, c;
+  sincospif(q, &s, &c);
+  return make_float2(fmaf(c, lo, s), fmaf(-s, lo, c));
 }
 
 // first of the k taps nearest y M = ih + fr: floor(y M - (k - 1)/2 + 1/2), mod M
@@ -121,16 +172,22 @@ __device__ __forceinline__ void move(const LocAxis& ax, int* ih, float* fr, floa
   *fr = f;
 }
 
-__global__ void __launch_bounds__(32 * kLocWarps, 4) localise_kernel(
+__global__ void __launch_bounds__(32 * kLocWarps, 5) localise_kernel(
     const float* __restrict__ P, float* __restrict__ out, int64_t items, LocAxis axx,
-    LocAxis axy, int n_iter, int taps_x, int taps_y, int vec4) {
+    LocAxis axy, int n_iter, int taps_x, int taps_y, int vec4, int tab) {
   __shared__ float sw[kLocWarps][4][kLocTaps];         // wx, dwx, wy, dwy of the taps
+  extern __shared__ float2 s_tab[];                    // (sin, cos)(pi k / My), k < 2 My, if `tab`
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   float* wx = sw[wib][0];
   float* dwx = sw[wib][1];
   float* wy = sw[wib][2];
   float* dwy = sw[wib][3];
   const int mx = axx.M, my = axy.M, nel = mx * my;
+  if (tab) {
+    for (int k = threadIdx.x; k < 2 * my; k += blockDim.x)
+      sincospif((float)k / (float)my, &s_tab[k].x, &s_tab[k].y);
+    __syncthreads();
+  }
   const int64_t warps = (int64_t)gridDim.x * kLocWarps;
   for (int64_t item = (int64_t)blockIdx.x * kLocWarps + wib; item < items; item += warps) {
     const float* tile = P + item * (int64_t)nel;
@@ -141,10 +198,12 @@ __global__ void __launch_bounds__(32 * kLocWarps, 4) localise_kernel(
       const float4* t4 = reinterpret_cast<const float4*>(tile);
       for (int i = lane; i < (nel >> 2); i += 32) {
         const float4 v = t4[i];
-        if (v.x > best) { best = v.x; bi = 4 * i; }
-        if (v.y > best) { best = v.y; bi = 4 * i + 1; }
-        if (v.z > best) { best = v.z; bi = 4 * i + 2; }
-        if (v.w > best) { best = v.w; bi = 4 * i + 3; }
+        const float m = fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w));   // NaN only if all four are
+        if (m > best) { best = m; bi = i; }
+      }
+      if (bi < nel) {                                  // the first of the four that is the maximum
+        const float4 v = t4[bi];
+        bi = 4 * bi + (v.x == best ? 0 : v.y == best ? 1 : v.z == best ? 2 : 3);
       }
     } else {
       for (int i = lane; i < nel; i += 32) {
@@ -175,7 +234,14 @@ __global__ void __launch_bounds__(32 * kLocWarps, 4) localise_kernel(
         wx[t] = w;
         dwx[t] = d;
       }
-      for (int t = lane; t < ky; t += 32) {
+      if (axy.fit && ky <= 16) {
+        float w, d;
+        dir_weight_pair(axy, ihy, fry, mod_m(axy, fy + (lane & 15)), lane, &w, &d);
+        if (lane < ky) {
+          wy[lane] = w;
+          dwy[lane] = d;
+        }
+      } else for (int t = lane; t < ky; t += 32) {
         float w = 1.f, d = 0.f;
         if (axy.fit) dir_weight(axy, ihy, fry, mod_m(axy, fy + t), &w, &d);
         wy[t] = w;
@@ -193,8 +259,8 @@ __global__ void __launch_bounds__(32 * kLocWarps, 4) localise_kernel(
         if (ty >= ky) { ty -= ky; ++tx; }
       }
       T = warp_sum_f(T);
-      Dx = warp_sum_f(Dx);
-      Dy = warp_sum_f(Dy);
+      if (axx.fit) Dx = warp_sum_f(Dx);
+      if (axy.fit) Dy = warp_sum_f(Dy);
       __syncwarp();
       if (axx.fit) move(axx, &ihx, &frx, Dx * axx.newton / T * (float)mx);
       if (axy.fit) move(axy, &ihy, &fry, Dy * axy.newton / T * (float)my);
@@ -203,6 +269,27 @@ __global__ void __launch_bounds__(32 * kLocWarps, 4) localise_kernel(
     // (regridding weights of both signs: compensated FP32 sums keep the cancellation exact
     // to about one rounding)
     CSum T;
+    // weight of beam B of the second axis: eight and more beams away sin(pi e) is the sum of two
+    // terms of which one is at most an eighth of the other, so nothing cancels; nearer by dir_weight
+    float2 fL, f1;
+    if (tab) {
+      fL = frac_angle(axy, (float)(2 * axy.n - 1), fry);
+      f1 = frac_angle(axy, 1.f, fry);
+    }
+    auto weight_y = [&](int B) {
+      int d;
+      float r, w, dw;
+      dir_d(axy, ihy, fry, B, &d, &r);
+      if (!tab || fabsf(r) < 8.f) {
+        dir_weight(axy, ihy, fry, B, &w, &dw);
+        return w;
+      }
+      int m2 = dir_m2(axy, d), m1 = d;
+      if (axy.pow2) m1 &= 2 * my - 1;
+      else { m2 += m2 < 0 ? 2 * my : 0; m1 += m1 < 0 ? 2 * my : 0; }
+      const float2 tL = s_tab[m2], t1 = s_tab[m1];
+      return fmaf(tL.x, fL.y, tL.y * fL.x) / (fmaf(t1.x, f1.y, t1.y * f1.x) * (float)my);
+    };
     if (axx.fit) {
       for (int c = 0; c < mx; c += kLocTaps) {
         for (int t = lane; t < kLocTaps && c + t < mx; t += 32) {
@@ -213,8 +300,8 @@ __global__ void __launch_bounds__(32 * kLocWarps, 4) localise_kernel(
         __syncwarp();
         const int na = mx - c < kLocTaps ? mx - c : kLocTaps;
         for (int B = lane; B < my; B += 32) {
-          float wB = 1.f, d;
-          if (axy.fit) dir_weight(axy, ihy, fry, B, &wB, &d);
+          float wB = 1.f;
+          if (axy.fit) wB = weight_y(B);
           else if (B != b0) continue;
           float s = 0.f;
           for (int A = 0; A < na; ++A) s = fmaf(wx[A], tile[(c + A) * my + B], s);
@@ -224,8 +311,8 @@ __global__ void __launch_bounds__(32 * kLocWarps, 4) localise_kernel(
       }
     } else {
       for (int B = lane; B < my; B += 32) {
-        float wB = 1.f, d;
-        if (axy.fit) dir_weight(axy, ihy, fry, B, &wB, &d);
+        float wB = 1.f;
+        if (axy.fit) wB = weight_y(B);
         else if (B != b0) continue;
         T.add(wB * tile[a0 * my + B]);
       }
@@ -270,10 +357,13 @@ extern "C" int fftbf_localise(fftbf_plan* p, const float* beams_dev, int64_t n_w
   cudaGetDevice(&prev);
   if (prev != p->device) cudaSetDevice(p->device);
   const int64_t items = n_windows * p->nfreq;
-  const int64_t blocks = std::min<int64_t>((items + kLocWarps - 1) / kLocWarps, (int64_t)p->nsm * 4);
-  localise_kernel<<<(unsigned)blocks, 32 * kLocWarps, 0, static_cast<cudaStream_t>(stream)>>>(
+  // two rounds of the resident CTAs, so that the SMs that finish first take more (120 -> 118 us)
+  const int64_t blocks = std::min<int64_t>((items + kLocWarps - 1) / kLocWarps, (int64_t)p->nsm * 10);
+  const int tab = ay.fit && ay.M >= 32 && ay.M <= kLocTab;
+  localise_kernel<<<(unsigned)blocks, 32 * kLocWarps, tab ? sizeof(float2) * 2 * ay.M : 0,
+                    static_cast<cudaStream_t>(stream)>>>(
       beams_dev, out_dev, items, ax, ay, n_iter, std::min(n_taps, p->mx), std::min(n_taps, p->my),
-      vec4);
+      vec4, tab);
   const cudaError_t e = cudaGetLastError();
   if (prev != p->device) cudaSetDevice(prev);
   if (e != cudaSuccess) return cuda_error(e, "fftbf_localise");

@@ -77,3 +77,29 @@ def test_localise_rejects_bad_taps():
             with pytest.raises(fb.FftbfError) as e:
                 fb.localise(plan, P, 1, out, n_iter=2, n_taps=bad)
             assert e.value.code == -1
+
+
+@pytest.mark.parametrize("nx,ny,mx,my", [(1, 16, 1, 31), (1, 16, 1, 32), (2, 20, 2, 41),      # direct, table
+                                         (1, 700, 1, 1500),
+                                         (1, 1024, 1, 2048), (1, 1024, 1, 2060)])             # last, direct
+def test_localise_final_sum_over_sizes(nx, ny, mx, my):
+    """The final sum with its N-S sines from the table (32 <= pad_y <= 2048) and from direct calls on
+    either side, powers of two and odd pads: the oracle's estimate of the same beams, within the
+    bounds of the other comparisons here."""
+    rng = np.random.default_rng(3)
+    nwin, nfreq = 3, 2
+    y0 = rng.random((nwin, nfreq))
+    B = np.arange(my) / my
+    row = np.abs(np.sum(np.exp(2j * np.pi * np.arange(ny) * (B[None, None, :, None] - y0[..., None, None])),
+                        axis=-1)) ** 2 / ny ** 2 + 0.05                 # one source over a floor
+    P = np.repeat(row[:, :, None, :], mx, axis=2).astype(np.float32)
+    P[:, :, 0] *= 1.5
+    dP = torch.from_numpy(P).cuda()
+    out = torch.full((nwin, nfreq, 3), float("nan"), device="cuda")
+    with fb.plan_create(nx, ny, mx, my, 1, nfreq, 8) as plan:
+        fb.localise(plan, dP, nwin, out, n_iter=5, n_taps=10)
+        fb.plan_sync(plan)
+    got = out.cpu().numpy()
+    ref = oracle.localise(P, nx, ny, n_iter=5, n_taps=10)
+    assert (np.abs((got[..., :2] - ref[..., :2] + 0.5) % 1.0 - 0.5) < 2e-6).all()
+    assert np.allclose(got[..., 2], ref[..., 2], rtol=1e-5)
