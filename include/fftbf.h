@@ -219,10 +219,12 @@ int fftbf_execute_host(fftbf_plan* plan, const uint8_t* volts_host, int64_t T,
 
 /*
  * Batches: several plans (arrays of different lattice sizes, channel counts and weights)
- * transformed by ONE persistent launch of the FP32 form. Work items are (array, window,
- * channel) taken from a device work queue, costliest arrays first; each array runs the
- * transform of its own shape, with a snapshots-per-step tile picked for it by timing the
- * candidates on the device at creation. Supported shapes (pad_x x pad_y, pad_y >= ny):
+ * transformed by as few persistent launches of the FP32 form as they allow, usually ONE: arrays
+ * whose items go through the feed covariance (see FFTBF_PREC_FP32) and the others run in launches
+ * of their own. Work items are (array, window, channel), costliest arrays first; an array of the
+ * second kind runs the transform of its own shape, its items taken from a device work queue, with
+ * a snapshots-per-step tile picked for it by timing the candidates on the device at creation.
+ * Supported shapes (pad_x x pad_y, pad_y >= ny):
  * 4x512, 8x128, 16x32, 2x1024, 1x2048, 3x256 (the N-S axis padded to twice the next
  * power of two of 256, 64, 16, 512, 1024, 128 feeds); others give FFTBF_EUNSUPPORTED.
  * The plans must outlive the batch, be on one device and not change precision.
@@ -239,10 +241,11 @@ fftbf_batch* fftbf_batch_create(fftbf_plan* const* plans, int n);
  */
 int fftbf_batch_execute(fftbf_batch* batch, const uint8_t* const* volts_dev, int64_t T,
                         float* const* beams_dev, void* stream);
-/* Snapshots per step the autotuner chose for plan i of the batch (>= 1), or < 0. */
+/* Snapshots per step of plan i of the batch (>= 1): the autotuner's choice, or 64 for an array that
+ * goes through the feed covariance; < 0 on error. */
 int fftbf_batch_tuned_steps(const fftbf_batch* batch, int i);
-/* CTAs of each batched launch: the launch's persistent grid (SMs x resident CTAs per SM);
- * work items beyond it are taken from the device queue in turn. */
+/* CTAs of the batched launch: the persistent grid (SMs x resident CTAs per SM; one CTA per SM, in
+ * pairs, when every array goes through the feed covariance); work items beyond it are taken in turn. */
 int fftbf_batch_grid(const fftbf_batch* batch);
 /* Free the batch (waits for its last launch). NULL is a no-op. */
 void fftbf_batch_destroy(fftbf_batch* batch);
@@ -255,7 +258,8 @@ void fftbf_batch_destroy(fftbf_batch* batch);
  * waits while no slot is free), copies them to the device, and whenever frames are staged
  * and a launch slot is free, transforms every staged frame in one persistent batched
  * launch (up to 64 frames; two launches may be in flight), so frames that arrive while
- * others are on the GPU join the next launch and their work overlaps. A frame's beams are
+ * others are on the GPU join the next launch and their work overlaps. (Frames that go through the
+ * feed covariance and frames that do not run in launches of their own.) A frame's beams are
  * bit-identical alone and in any mix. Lattice shapes: those of fftbf_batch_create.
  * Host buffers must stay valid until the frame completes; pinned memory lets copies and
  * transforms overlap.
