@@ -40,9 +40,9 @@
 // off-diagonal tile the MMAs read 64 KB, the producers write 32 KB and the staging moves 32 KB:
 // about 128 bytes per cycle), and between tiles the epilogue, whose products keep the FMA pipe
 // busy for ~1000 cycles per half. Measured on a GB300 (before: the FFT kernels): 4x256, 2
-// polarisations, 4096 windows x channels of 768 snapshots 8.57 -> 5.18 ms (10.6 us per tile; the
-// MMAs alone would need 3.0 ms); 16 such items 608 -> 102 us; 8x64 with complex gains, 2048 items
-// of 512 snapshots 3.44 -> 0.92 ms; 3x37 onto 5x73 beams, 360 items of 100 snapshots 1267 -> 152
+// polarisations, 4096 windows x channels of 768 snapshots 8.57 -> 5.20 ms (10.6 us per tile; the
+// MMAs alone would need 3.0 ms); 16 such items 608 -> 104 us; 8x64 with complex gains, 2048 items
+// of 512 snapshots 3.44 -> 0.90 ms; 3x37 onto 5x73 beams, 360 items of 100 snapshots 1267 -> 143
 // us. Error against FP64 2.5e-8 (2-norm), before 1e-7 to 6e-7.
 // Every sum is taken in a fixed order that depends on the item alone, so an item's beams are
 // bit-identical whatever else the launch carries.

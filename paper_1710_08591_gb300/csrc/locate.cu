@@ -22,7 +22,9 @@
 // with every sine computed, a compare and two selects per beam in the search for the maximum and four
 // CTAs per SM (3870 warp instructions per item); 132 us with the table, the search by four beams and
 // the two sines of a tap in two lanes; 118 us at five CTAs per SM (48 registers, no spills; six
-// spill). 8192 items of 8x128: 24 us.
+// spill); 114 us with the next beam of the final sum loaded under this one's weight, 2048 items of
+// 1x2048 33 to 25 us. 8192 items of 8x128: 24 us. The weights as a called function instead of five
+// inlined copies (a tenth of the stalls are instruction fetches) took 124 us.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -310,11 +312,15 @@ __global__ void __launch_bounds__(32 * kLocWarps, 5) localise_kernel(
         __syncwarp();
       }
     } else {
+      const float* row = tile + a0 * my;
+      float p = lane < my ? row[lane] : 0.f;
       for (int B = lane; B < my; B += 32) {
+        const float pB = p;                              // the next beam's load under this one's weight
+        if (B + 32 < my) p = row[B + 32];
         float wB = 1.f;
         if (axy.fit) wB = weight_y(B);
         else if (B != b0) continue;
-        T.add(wB * tile[a0 * my + B]);
+        T.add(wB * pB);
       }
     }
     const float Tsum = warp_sum_c(T);
