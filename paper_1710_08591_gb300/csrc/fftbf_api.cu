@@ -98,7 +98,6 @@ fftbf_plan* fftbf_plan_create(int nx, int ny, int pad_x, int pad_y, int npol, in
   if (e == cudaSuccess) e = cudaMalloc(&p->d_w, sizeof(float2) * nant);
   if (e == cudaSuccess) e = cudaMalloc(&p->d_ex, sizeof(float2) * pad_x * nx);
   if (e == cudaSuccess) e = cudaMalloc(&p->d_tw, sizeof(float2) * pad_y);
-  if (e == cudaSuccess) e = cudaMalloc(&p->d_cw, sizeof(float4) * (pad_y + pad_x));
   if (e == cudaSuccess) e = cudaMalloc(&p->d_err, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(p->d_err, 0, sizeof(int));
   if (e == cudaSuccess) {
@@ -111,13 +110,26 @@ fftbf_plan* fftbf_plan_create(int nx, int ny, int pad_x, int pad_y, int npol, in
     for (int i = 0; i < nant; ++i) p->real_w = p->real_w && p->h_w[2 * i + 1] == 0.f;
     e = cudaMemcpy(p->d_w, p->h_w.data(), sizeof(float2) * nant, cudaMemcpyHostToDevice);
   }
+  // the table of the covariance route, for plans that take it in some precision (a rule on sizes);
+  // without it the route is refused. The rule only asks whether there is a table.
+  if (e == cudaSuccess) {
+    BeamArgs a{};
+    a.nx = nx; a.ny = ny; a.mx = pad_x; a.my = pad_y;
+    a.npol = npol; a.nfreq = nfreq; a.n_int = n_int;
+    a.nyf = std::min(ny, pad_y);
+    a.real_w = p->real_w ? 1 : 0;
+    float4 here;
+    a.cw = &here;
+    if (corr_preferred(a) || (tc_supported(nx, ny, pad_x, pad_y) && corr_preferred(a, true)))
+      e = cudaMalloc(&p->d_cw, sizeof(float4) * (pad_y + pad_x));
+  }
   if (e != cudaSuccess) {
     cuda_error(e, "fftbf_plan_create");
     fftbf_destroy(p);
     return nullptr;
   }
   if (build_tables(nx, pad_x, pad_y, p->d_ex, p->d_tw, 0) != FFTBF_OK ||
-      build_corr_table(pad_x, pad_y, p->d_cw, 0) != FFTBF_OK ||
+      (p->d_cw && build_corr_table(pad_x, pad_y, p->d_cw, 0) != FFTBF_OK) ||
       (e = cudaDeviceSynchronize()) != cudaSuccess) {
     if (e != cudaSuccess) cuda_error(e, "plan tables");
     fftbf_destroy(p);
