@@ -195,6 +195,13 @@ __device__ __forceinline__ void tma_volts(uint32_t dst, const CUtensorMap* map, 
       : "memory");
 }
 
+// A tensor map in global memory was written by a copy (generic proxy): before its first use by TMA
+// the writes are acquired for the tensor-map proxy, or a descriptor cached from the table's earlier
+// contents could be used. Maps in kernel parameters need no fence.
+__device__ __forceinline__ void acquire_map(const CUtensorMap* map) {
+  asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;\n" ::"l"(map) : "memory");
+}
+
 // The first `cnt` of 16 bytes at any address: aligned words where they lie inside
 // [begin, end), single bytes at the ends of the buffer.
 __device__ __noinline__ uint4 load16_any(const uint8_t* p, int cnt, const uint8_t* begin,
@@ -840,8 +847,11 @@ __device__ __forceinline__ void stage_volts(const CorrParams& P, unsigned char* 
   int64_t n = 0;                                       // stages issued
   int job = 0;
   bool ok = true;
+  const CorrJob* last = nullptr;
   for (int64_t item = pair; item < P.total && ok; item += npairs) {
     const CorrJob& J = find_job(P, item, job);
+    if (P.table && &J != last) acquire_map(&J.map);
+    last = &J;
     const int nt = J.nt, np = J.np, npol = J.a.npol, nch = J.nch;
     const int64_t jw = (item - J.item0) / J.a.nfreq;
     const int f = (int)(item - J.item0 - jw * J.a.nfreq), t0 = (int)(jw * J.a.n_int);

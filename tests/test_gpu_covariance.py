@@ -167,3 +167,61 @@ def test_server_frames_through_the_covariance():
         assert np.array_equal(o[None], _batch([(s, v, None)], n_int, 1)[0])
     for p in plans:
         p.close()
+
+
+def test_batch_on_alternating_buffers():
+    """One batch on two sets of buffers of different contents in turn: each call rewrites the job
+    table and its tensor maps in place, and every array's beams are its own buffers'."""
+    n_int, nwin = 320, 2
+    shapes = [(4, 256, 4, 512), (8, 64, 8, 128), (16, 16, 16, 32)]
+    T = nwin * n_int
+    plans = [fb.plan_create(*s, 2, 2, n_int) for s in shapes]
+    sets = []
+    for k in range(2):
+        g = torch.Generator(device="cuda")
+        g.manual_seed(40 + k)
+        vs = [torch.randint(0, 256, (T * 2 * 2 * s[0] * s[1],), dtype=torch.uint8, device="cuda", generator=g)
+              for s in shapes]
+        want = [torch.empty((nwin, 2, s[2], s[3]), device="cuda") for s in shapes]
+        for p, v, o in zip(plans, vs, want):
+            fb.execute(p, v, T, o)
+        sets.append((vs, want, [torch.empty_like(o) for o in want]))
+    st = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with fb.batch_create(plans) as b:
+        for turn in range(24):
+            vs, want, outs = sets[turn % 2]
+            for o in outs:
+                o.fill_(float("nan"))
+            torch.cuda.synchronize()
+            fb.batch_execute(b, vs, T, outs, st if turn % 3 else None)
+            torch.cuda.synchronize()
+            for o, w in zip(outs, want):
+                assert torch.equal(o, w), turn
+    for p in plans:
+        fb.plan_sync(p)
+        p.close()
+
+
+def test_server_ticks_reuse_slots_for_other_lattices():
+    """Rounds of frames through few slots: every tick rewrites its table with other slots, lattices
+    and contents, and each frame's beams are those of its own voltages."""
+    n_int, nf = 320, 2
+    shapes = [(8, 64, 8, 128), (4, 256, 4, 512), (16, 16, 16, 32)]
+    plans = [fb.plan_create(*s, 2, nf, n_int) for s in shapes]
+    rng = np.random.default_rng(9)
+    with fb.server_create(plans, 16 << 20) as sv:
+        for _ in range(6):
+            frames, outs, which = [], [], rng.integers(3, size=8)
+            for k in which:
+                s = shapes[k]
+                frames.append(rng.integers(0, 256, n_int * nf * 2 * s[0] * s[1], dtype=np.uint8))
+                outs.append(np.full((nf, s[2], s[3]), np.nan, np.float32))
+                fb.server_submit(sv, int(k), frames[-1], outs[-1])
+            fb.server_wait(sv)
+            for k, v, o in zip(which, frames, outs):
+                want = torch.empty((1,) + o.shape, device="cuda")
+                fb.execute(plans[k], torch.from_numpy(v).cuda(), n_int, want)
+                assert np.array_equal(o, want.cpu().numpy()[0])
+    for p in plans:
+        p.close()
