@@ -320,6 +320,7 @@ static void fill_args(const fftbf_plan* p, BeamArgs& a) {
   a.real_w = p->real_w ? 1 : 0;
   a.cw = p->d_cw;
   a.err = p->d_err;
+  a.w_exp = p->w_exp;
 }
 
 static int launch_jobs(fftbf_batch* bb, int64_t total, cudaStream_t st) {

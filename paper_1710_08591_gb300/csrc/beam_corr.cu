@@ -11,7 +11,9 @@
 // pattern k: the subnormals and the first binade are one linear scale of 2^-9), and the
 // tensor cores sum their products in FP32: R is exact while 128 snapshots <= 2^24. So one
 // FP8 product per pair replaces the FP32 transform of every snapshot; the weights and the
-// transform are applied once per window, in FP32, to exact sums.
+// transform are applied once per window, to exact sums: in FP32 with every product's rounding
+// error kept, V in fixed point of about 2^-38 of the largest product, the transform in two floats,
+// because a weak beam beside a strong source is a small difference of large terms.
 //
 // Work split: one pair of CTAs (a cluster, tcgen05 cta_group::2) owns a work item (window,
 // channel) and walks the upper-triangle tiles of R, 256 feeds x up to 256 feeds, one tile in
@@ -20,9 +22,10 @@
 // leaves the SM. Feeds are held in slots ix * nyp + iy, nyp = ny rounded up to a multiple of
 // 16 (zeros between), so a group of 16 slots lies in one E-W row. Roles (18 of 20 warps per CTA):
 //   warps 0-7    epilogue: weights x covariance, summed along the diagonals of the tile,
-//                added to V in shared memory; after the last tile the transform of V to beams;
+//                added to V in shared memory (each warp at its own pace); after the last tile the
+//                transform of V to beams;
 //   warps 8-15   producers: voltages of this CTA's 128 row slots and its half of the column
-//                slots, 32 snapshots per chunk, nibbles to e4m3 (both MN-major operands);
+//                slots, 64 snapshots per stage, nibbles to e4m3 (both MN-major operands);
 //   warp 17      one thread stages the voltages with TMA (64 snapshots x 128 feeds a tile);
 //   warps 16, 18 one thread each of the pair's first CTA issue the MMAs of the real and of the
 //                imaginary half: per 32 snapshots
@@ -36,16 +39,18 @@
 // cores busy), so the real products of the next tile run while the epilogue reads this tile's
 // imaginary half, ahead by as many stages as the operand ring holds. Every wait is bounded by
 // one second of device time.
-// What bounds it: shared-memory bandwidth and the tensor cores together (per stage of an
+// What bounds it: the producers' integer unpacking and shared memory beside the MMAs (per stage of an
 // off-diagonal tile the MMAs read 64 KB, the producers write 32 KB and the staging moves 32 KB:
-// about 128 bytes per cycle), and between tiles the epilogue, whose products keep the FMA pipe
-// busy for ~1000 cycles per half. Measured on a GB300 (before: the FFT kernels): 4x256, 2
-// polarisations, 4096 windows x channels of 768 snapshots 8.57 -> 5.20 ms (10.6 us per tile; the
-// MMAs alone would need 3.0 ms); 16 such items 608 -> 104 us; 8x64 with complex gains, 2048 items
-// of 512 snapshots 3.44 -> 0.90 ms; 3x37 onto 5x73 beams, 360 items of 100 snapshots 1267 -> 143
-// us. Error against FP64 2.5e-8 (2-norm), before 1e-7 to 6e-7.
-// Every sum is taken in a fixed order that depends on the item alone, so an item's beams are
-// bit-identical whatever else the launch carries.
+// about 128 bytes per cycle), and between tiles the epilogue, about 4500 cycles per half with real
+// weights: a third its products, a third the gather of the lags. Measured on a GB300 (the FFT
+// kernels; this one with products and sums rounded to FP32; this one): 4x256, 2 polarisations,
+// 4096 windows x channels of 768 snapshots 8.57, 5.20, 6.09 ms (the MMAs alone would need 3.3 ms, 540
+// tiles of 6.1 us in turn); 16 such items 608, 104, 119 us; 8x64 with complex gains, 2048 items of 512
+// snapshots 3.44, 0.90, 1.17 ms; 3x37 onto 5x73 beams, 360 items of 100 snapshots 1267, 143, 139 us.
+// Largest error of a beam beside a source of amplitude 7 over noise of 0.3, 4x256 with half-sine
+// weights: 2e-6, 1e-4, 6e-8.
+// An item's sums are whole numbers or taken in an order that depends on the item alone, so its
+// beams are bit-identical whatever else the launch carries.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -68,7 +73,8 @@ constexpr int TILE = 128 * KS;           // one operand component: 128 slots x 6
 constexpr int STAGE = 4 * TILE;          // rows re, rows im, columns re, columns im
 constexpr int LBO = 1024, SBO = 128;     // MN-major: 8 snapshots apart, 16 slots apart
 constexpr int VMAX = 2048;               // entries of V (E-W separations x N-S lags)
-constexpr int DS = 72;                   // floats per staged diagonal (8 x 8, conflict-free gather)
+constexpr int DS = 72;                   // pairs per staged diagonal (8 x 8, conflict-free gather)
+constexpr float GRID = 12582912.f;       // 1.5 2^23: sums started here are whole numbers
 constexpr int MAXNS = 6, MAXNR = 3;
 constexpr int RAW = KS * 128;            // staged voltages of one operand: 64 snapshots x 128 feeds
 constexpr uint64_t WAIT_NS = 1000000000ull;
@@ -169,20 +175,16 @@ __device__ __forceinline__ bool bar_epi_all(bool ok) {
 // TMEM -> registers, 16 lanes x 8 NB columns: thread t gets, for every 8-column block n,
 // r[4n], r[4n+1] = row t/4, columns 8n + 2(t%4), +1 and r[4n+2], r[4n+3] = row t/4 + 8.
 template <int NB> __device__ __forceinline__ void tmem_ld16x256(uint32_t taddr, uint32_t* r);
+template <> __device__ __forceinline__ void tmem_ld16x256<1>(uint32_t taddr, uint32_t* r) {
+  asm volatile("tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr));
+}
 template <> __device__ __forceinline__ void tmem_ld16x256<2>(uint32_t taddr, uint32_t* r) {
   asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
                  "=r"(r[6]), "=r"(r[7])
                : "r"(taddr));
-}
-template <> __device__ __forceinline__ void tmem_ld16x256<4>(uint32_t taddr, uint32_t* r) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
-      "%15}, [%16];\n"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
 }
 // TMA tile: `rows` of 128 bytes from feed x of channel f, time t on, all polarisations (snapshots in
 // order), 128-byte swizzle; zeros past the feeds and past the last sample.
@@ -282,11 +284,6 @@ __device__ __forceinline__ Cdd dd_cmul(Cdd a, float4 w) {
   return dd_add(p, q);
 }
 __device__ __forceinline__ Cdd dd_zero() { return Cdd{make_float2(0.f, 0.f), make_float2(0.f, 0.f)}; }
-__device__ __forceinline__ void dd_acc(Cdd& a, float2 x) {
-  const float2 s = cadd(a.h, x), t = csub(s, a.h);
-  a.l = cadd(a.l, cadd(csub(a.h, csub(s, t)), csub(x, t)));
-  a.h = s;
-}
 
 // The job of a work item; k: the job of this role's last item (items only grow).
 __device__ __forceinline__ const CorrJob& find_job(const CorrParams& p, int64_t item, int& k) {
@@ -309,10 +306,10 @@ __device__ __forceinline__ int tile_cols(int np, int J) {
 }
 
 // What the epilogue needs of a job, in registers.
-struct JobRegs { int nx, ny, nyp, np, nt, mx, mode; };
+struct JobRegs { int nx, ny, nyp, np, nt, mx, mode; float rscale, lscale; };
 
 struct Lay {                             // shared-memory offsets (bytes)
-  int ring, raw, w, v, stg, sl, tab, total;
+  int ring, raw, w, v, stg, tab, total;
 };
 __host__ __device__ inline Lay lay_of(const CorrSizes& s) {
   Lay L;
@@ -323,36 +320,60 @@ __host__ __device__ inline Lay lay_of(const CorrSizes& s) {
   L.w = take(s.wslots * 4 * (s.cplx ? 2 : 1));
   L.v = take(s.vlen * 16);
   L.stg = take(s.stg * 8 * 4);           // 8 warps; also the transform's buffer
-  L.sl = take(s.slice * 8 * 4);
   L.tab = take(s.tab * 16);
   L.total = o;
   return L;
 }
 
-// floats of one warp's staged diagonals of one row run (with a zero row each side) and of all its
-// row runs, and of its lag sums: (4 / G) (16 / CR) run pairs of 8 (G + CR) lags
-__host__ __device__ constexpr int stg_run(int G, int CR) { return (G + CR + 1) * DS + 8; }
-__host__ __device__ constexpr int stg_floats(int G, int CR) { return (4 / G) * stg_run(G, CR); }
-__host__ __device__ constexpr int slice_floats(int G, int CR) { return (4 / G) * (16 / CR) * 8 * (G + CR); }
+// Floats of one warp's staged diagonals, (whole, rest) pairs of c components: the G + 1 of a step, the
+// last one copied to the front for the next, or where there is room (c = 1) and several steps a ring
+// of 2 G, its first one held behind the last as well so that a step's lie in order.
+__host__ __device__ constexpr int stg_rows(int G, int CR, int c) { return c == 1 && CR > G ? 2 * G + 1 : G + 1; }
+__host__ __device__ constexpr int stg_floats(int G, int CR, int c) { return 2 * c * (4 / G) * stg_rows(G, CR, c) * DS; }
+
+// a x, exactly: the product and its rounding error with the sign changed (nx = -x)
+__device__ __forceinline__ float2 mul_exact(float2 a, float2 x, float2 nx, float2& nerr) {
+  const float2 p = __fmul2_rn(a, x);
+  nerr = __ffma2_rn(a, nx, p);
+  return p;
+}
+// grid += a x in whole numbers; returns what that rounds away (|.| <= 1/2)
+__device__ __forceinline__ float2 fma_grid(float2 a, float2 x, float2& grid) {
+  const float2 t = __ffma2_rn(a, x, grid), d = csub(grid, t);
+  grid = t;
+  return __ffma2_rn(a, x, d);
+}
 
 // ---- epilogue of a tile, one warp: 32 rows x 128 columns of one half (real or imaginary), or with
 // complex weights of both. Slots are in runs of G 8-row groups (rows) and CR 8-column groups
 // (columns) that each lie in one E-W row. A thread holds, of every 8 x 8 block, row r = lane/4 and
 // two adjacent columns; it sums w_a R_ab w_b of the blocks on one block diagonal, d = j - i, in
-// registers (bound by the FMA pipe: one packed multiply and one FMA per two elements); the
-// diagonals go to shared memory and each lane gathers lags b - a: slice[u], u = lag + 8G - 1.
+// registers. A weak beam beside a strong source is a small difference of these products, so none of
+// their bits is dropped: the weights are scaled by powers of two so that no product exceeds 2^19,
+// each is added to a sum that starts at 1.5 2^23 and so takes whole numbers only, and what that
+// leaves (an exact difference) goes to a second sum, with the products' own rounding errors: seven
+// packed instructions per two elements where rounded products took two, and 37 for 9 with complex
+// weights, whose z = w_b^* R is put on such a grid first. Both sums of G diagonals at a time go to
+// shared memory, each lane gathers one lag b - a of them and adds it to V in fixed point, whole
+// numbers and 2^-19 (1 / lscale) units in two words: integer additions, so V does not depend on their order and
+// the warps need no barrier between tiles.
 template <int G, int CR, bool CPLX>
-__device__ __forceinline__ void corr_phase(uint32_t tacc, int q, int h, int cols, int row0,
-                                           int col0, float scale, const float* ws, int wslots,
-                                           float* stg, float* sl, bool diag, uint32_t drained,
-                                           uint32_t drained2, int lane) {
-  constexpr int NU = 8 * (G + CR);                     // lags of a run pair, one spare
-  constexpr int SG = 4 / G, NST = stg_run(G, CR), CST = stg_floats(G, CR);
-  constexpr int JB = CPLX ? 2 : G;                     // 8-column blocks per load
+__device__ __forceinline__ void corr_phase(uint32_t tacc, int cols, int row0, int col0, float scale,
+                                           int ws0, int wslots, int stg0, int v0, int nv, int half,
+                                           int nx, int ny, int nyp, int mx, float lscale, bool diag,
+                                           uint32_t drained, uint32_t drained2) {
+  extern __shared__ __align__(1024) unsigned char smem_corr[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = warp & 3, h = warp >> 2;
+  const float* ws = reinterpret_cast<const float*>(smem_corr + ws0);
+  constexpr int NC = CPLX ? 2 : 1;                     // staged components: re, im
+  constexpr int SG = 4 / G, ROWS = stg_rows(G, CR, NC);
+  constexpr bool RING = ROWS > G + 1;
+  constexpr int NST = ROWS * DS, CST = SG * NST;       // pairs of a row run, of a component
+  float2* stg = reinterpret_cast<float2*>(smem_corr + stg0 + warp * 4 * stg_floats(G, CR, NC));
+  int* v = reinterpret_cast<int*>(smem_corr + v0);
+  constexpr int JB = CPLX ? 1 : 2;                     // 8-column blocks per load
   const int r = lane >> 2, c2 = 2 * (lane & 3);
-  int goff[8];                                         // gather of lag u = lane: one term per r
-#pragma unroll
-  for (int rr = 0; rr < 8; ++rr) goff[rr] = ((lane + 1 + rr) >> 3) * DS + 8 * rr + ((lane + 1 + rr) & 7);
+  const float2 grid0 = make_float2(GRID, GRID), zero = make_float2(0.f, 0.f);
   float wr[4], wi[4];                                  // rows 8 i + r of the warp's 32
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -361,6 +382,18 @@ __device__ __forceinline__ void corr_phase(uint32_t tacc, int q, int h, int cols
     wi[i] = CPLX ? ws[wslots + s] * scale : 0.f;
   }
   const float rs = CPLX && diag ? 0.5f : 1.f;          // complex: real half of a diagonal tile once
+  // gather of lag u = 8 G step + ul: one term per r, c = (u + 1 + r) mod 8 of staged diagonal
+  // (u + 1 + r) / 8
+  const int ul = lane & (8 * G - 1), sgl = G == 4 ? 0 : lane >> 4;
+  const float2* gat[8];
+#pragma unroll
+  for (int rr = 0; rr < 8; ++rr) {
+    const int k = ul + 1 + rr;
+    gat[rr] = stg + sgl * NST + (k >> 3) * DS + 8 * rr + (k & 7);
+  }
+  float2* put = stg + 2 * lane;
+  const int rowl = row0 + 32 * q + 8 * G * sgl;        // first slot of this lane's row run
+  const int ia = rowl / nyp, ya = rowl - ia * nyp;
   // the accumulators go back to the MMAs once the last of them is in registers
   const int runs = cols > 128 * h ? min(16 / CR, (cols - 128 * h + 8 * CR - 1) / (8 * CR)) : 0;
   auto release = [&]() {
@@ -372,23 +405,80 @@ __device__ __forceinline__ void corr_phase(uint32_t tacc, int q, int h, int cols
     }
   };
   if (runs == 0) release();
+  // Lags ul + 8 G step of a step's staged diagonals (rows from `at` on) to V: iy_a - iy_b = lam, and
+  // -lam of the conjugate; kap -1 where no feeds are.
+  auto gather = [&](int at, int lam, int kap) {
+    __syncwarp();
+    float2 x[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      float2 t[8];
+#pragma unroll
+      for (int rr = 0; rr < 8; ++rr) t[rr] = gat[rr][c * CST + at * DS];
+      x[c] = cadd(cadd(cadd(t[0], t[1]), cadd(t[2], t[3])), cadd(cadd(t[4], t[5]), cadd(t[6], t[7])));
+    }
+    __syncwarp();
+    const bool mir = lam < 0;
+    if (mir) {
+      lam = -lam;
+      kap = kap > 0 ? mx - kap : kap;
+    }
+    if (kap < 0 || lam >= ny) return;
+    int* o = v + kap * ny + lam;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const bool im = CPLX ? c == 1 : half == 1;
+      if (im && mir) x[c] = neg2(x[c]);
+      atomicAdd(o + (im ? 2 * nv : 0), __float2int_rn(x[c].x));
+      atomicAdd(o + (im ? 3 * nv : nv), __float2int_rn(x[c].y * lscale));
+    }
+  };
 #pragma unroll 1
   for (int run = 0; run < runs; ++run) {
     const int cc = 128 * h + 8 * CR * run;             // first column of the run in the tile
-    float2 acc[SG][G], aci[SG][G];
+    const int ib = (col0 + cc) / nyp, yb = col0 + cc - ib * nyp;
+    int kap = (ia - ib) % mx;
+    kap = ia < nx && ib < nx ? (kap < 0 ? kap + mx : kap) : -1;
+    float2 acc[SG][G], low[SG][G], aci[SG][G], lowi[SG][G];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) acc[i / G][i % G] = aci[i / G][i % G] = make_float2(0.f, 0.f);
-    float* so = stg + DS + 2 * lane;                   // staged row 1 (d = -(G-1)) of this thread
-#pragma unroll 1
-    for (int j0 = 0; j0 < CR; j0 += G, so += G * DS) {
+    for (int i = 0; i < 4; ++i) {
+      acc[i / G][i % G] = aci[i / G][i % G] = grid0;
+      low[i / G][i % G] = lowi[i / G][i % G] = zero;
+    }
+    const int lam0 = ya - yb - ul + 8 * G - 1;
+    auto stage = [&](int sg, int row, float2 a, float2 l, float2 ai, float2 li) {
+      float2* o = put + sg * NST + row * DS;
+      a = csub(a, grid0);
+      *reinterpret_cast<float4*>(o) = make_float4(a.x, l.x, a.y, l.y);
+      if constexpr (CPLX) {
+        ai = csub(ai, grid0);
+        *reinterpret_cast<float4*>(o + CST) = make_float4(ai.x, li.x, ai.y, li.y);
+      }
+    };
+    auto stage_zero = [&](int row) {                   // before the first diagonal and after the last
+#pragma unroll
+      for (int sg = 0; sg < SG; ++sg) stage(sg, row, grid0, zero, grid0, zero);
+    };
+    auto carry = [&]() {
+#pragma unroll
+      for (int k = 0; k < SG * NC; ++k) {
+        float2* o = put + k * NST;                     // CST = SG NST
+        *reinterpret_cast<float4*>(o) = *reinterpret_cast<const float4*>(o + G * DS);
+      }
+    };
+    stage_zero(0);
+#pragma unroll(CPLX ? (CR > G ? 2 : 1) : CR / G)
+    for (int j0 = 0; j0 < CR; j0 += G) {
+      const int at = RING ? j0 & G : 0;                // row before the step's first diagonal
+      if (!RING && CR > G && j0 > 0) carry();
 #pragma unroll
       for (int jb = 0; jb < G; jb += JB) {
-        uint32_t v[2][4 * JB], vi[2][4 * JB];          // 32 rows x 8 JB columns
+        uint32_t w[2][4 * JB], wim[2][4 * JB];         // 32 rows x 8 JB columns
         const uint32_t ta = tacc + ((uint32_t)(32 * q) << 16) + cc + 8 * (j0 + jb);
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
-          tmem_ld16x256<JB>(ta + ((uint32_t)(16 * i) << 16), v[i]);
-          if (CPLX) tmem_ld16x256<JB>(ta + 256 + ((uint32_t)(16 * i) << 16), vi[i]);
+          tmem_ld16x256<JB>(ta + ((uint32_t)(16 * i) << 16), w[i]);
+          if (CPLX) tmem_ld16x256<JB>(ta + 256 + ((uint32_t)(16 * i) << 16), wim[i]);
         }
         float2 br[JB], bi[JB];
 #pragma unroll
@@ -402,243 +492,67 @@ __device__ __forceinline__ void corr_phase(uint32_t tacc, int q, int h, int cols
 #pragma unroll
         for (int j = 0; j < JB; ++j) {
           const int jj = jb + j, done = (jj + 1) % G;  // block diagonal j0 + jj - (G - 1) completes
+          const float2 nb = CPLX ? neg2(bi[j]) : neg2(br[j]);
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
-            const uint32_t* x = &v[i >> 1][4 * j + 2 * (i & 1)];
+            const uint32_t* x = &w[i >> 1][4 * j + 2 * (i & 1)];
             const float2 R = make_float2(__uint_as_float(x[0]), __uint_as_float(x[1]));
             const int sg = i / G, d = (jj - i % G + G) % G;
-            const float2 ar = make_float2(wr[i], wr[i]);
+            const float2 ar = make_float2(wr[i], wr[i]), na = make_float2(-wr[i], -wr[i]);
             if constexpr (!CPLX) {
-              acc[sg][d] = __ffma2_rn(__fmul2_rn(R, br[j]), ar, acc[sg][d]);
+              float2 ne;
+              const float2 p = mul_exact(R, br[j], nb, ne);
+              const float2 l = fma_grid(p, ar, acc[sg][d]);
+              low[sg][d] = cadd(low[sg][d], __ffma2_rn(ne, na, l));
             } else {                                   // w_a w_b^* (R + i X)
-              const float2 ai = make_float2(wi[i], wi[i]), na = make_float2(-wr[i], -wr[i]);
-              const uint32_t* y = &vi[i >> 1][4 * j + 2 * (i & 1)];
+              const float2 ai = make_float2(wi[i], wi[i]), nai = make_float2(-wi[i], -wi[i]);
+              const uint32_t* y = &wim[i >> 1][4 * j + 2 * (i & 1)];
               const float2 X = make_float2(__uint_as_float(y[0]), __uint_as_float(y[1]));
               const float2 S = __fmul2_rn(R, make_float2(rs, rs));
-              const float2 pr = __ffma2_rn(ai, bi[j], __fmul2_rn(ar, br[j]));
-              const float2 pi = __ffma2_rn(na, bi[j], __fmul2_rn(ai, br[j]));
-              acc[sg][d] = __ffma2_rn(make_float2(-pi.x, -pi.y), X, __ffma2_rn(pr, S, acc[sg][d]));
-              aci[sg][d] = __ffma2_rn(pr, X, __ffma2_rn(pi, S, aci[sg][d]));
+              float2 zr = grid0, zi = grid0;
+              const float2 zrl = cadd(fma_grid(S, br[j], zr), fma_grid(X, bi[j], zr));
+              const float2 zil = cadd(fma_grid(X, br[j], zi), fma_grid(S, nb, zi));
+              zr = csub(zr, grid0);
+              zi = csub(zi, grid0);
+              float2 l = cadd(fma_grid(zr, ar, acc[sg][d]), fma_grid(zi, nai, acc[sg][d]));
+              low[sg][d] = cadd(low[sg][d], __ffma2_rn(zil, nai, __ffma2_rn(zrl, ar, l)));
+              l = cadd(fma_grid(zi, ar, aci[sg][d]), fma_grid(zr, ai, aci[sg][d]));
+              lowi[sg][d] = cadd(lowi[sg][d], __ffma2_rn(zrl, ai, __ffma2_rn(zil, ar, l)));
             }
           }
 #pragma unroll
           for (int sg = 0; sg < SG; ++sg) {
-            *reinterpret_cast<float2*>(so + sg * NST + jj * DS) = acc[sg][done];
-            acc[sg][done] = make_float2(0.f, 0.f);
-            if constexpr (CPLX) {
-              *reinterpret_cast<float2*>(so + CST + sg * NST + jj * DS) = aci[sg][done];
-              aci[sg][done] = make_float2(0.f, 0.f);
-            }
+            stage(sg, at + 1 + jj, acc[sg][done], low[sg][done], aci[sg][done], lowi[sg][done]);
+            if (RING && jj == G - 1 && at == G) stage(sg, 0, acc[sg][done], low[sg][done], aci[sg][done], lowi[sg][done]);
+            acc[sg][done] = aci[sg][done] = grid0;
+            low[sg][done] = lowi[sg][done] = zero;
           }
         }
       }
+      gather(at, lam0 - 8 * j0, kap);
     }
-#pragma unroll
-    for (int sg = 0; sg < SG; ++sg)
-#pragma unroll
-      for (int e = 1; e < G; ++e) {                    // diagonals CR - G + 1 .. CR - 1
-        *reinterpret_cast<float2*>(so + sg * NST + (e - 1) * DS) = acc[sg][e % G];
-        if constexpr (CPLX) *reinterpret_cast<float2*>(so + CST + sg * NST + (e - 1) * DS) = aci[sg][e % G];
-      }
-    __syncwarp();
-    // lag u - 8G + 1 = 8 d + c - r: one term per r, from staged row (u + 1 + r) / 8
+    constexpr int AT = RING ? CR & G : 0;
+    if (!RING) carry();
 #pragma unroll
     for (int sg = 0; sg < SG; ++sg) {
-      float* so_sl = sl + (sg * (16 / CR) + run) * NU;
 #pragma unroll
-      for (int ub = 0; ub < NU; ub += 32) {            // the last lag is a spare, always zero
-#pragma unroll
-        for (int c = 0; c < (CPLX ? 2 : 1); ++c) {
-          const float* p = stg + c * CST + sg * NST + (ub / 8) * DS;
-          float x[8];
-#pragma unroll
-          for (int rr = 0; rr < 8; ++rr) x[rr] = p[goff[rr]];
-          so_sl[c * slice_floats(G, CR) + ub + lane] =
-              ((x[0] + x[1]) + (x[2] + x[3])) + ((x[4] + x[5]) + (x[6] + x[7]));
-        }
-      }
+      for (int e = 1; e < G; ++e)                      // diagonals CR - G + 1 .. CR - 1
+        stage(sg, AT + e, acc[sg][e % G], low[sg][e % G], aci[sg][e % G], lowi[sg][e % G]);
     }
-    __syncwarp();
+    stage_zero(AT + G);
+    gather(AT, lam0 - 8 * CR, kap);
   }
 }
-// The zero rows either side of a warp's staged diagonals.
-template <int G, int CR>
-__device__ __forceinline__ void corr_zero_rows(float* stg, int comps, int lane) {
-  for (int k = 0; k < comps * (4 / G); ++k) {
-    float* p = stg + (k / (4 / G)) * stg_floats(G, CR) + (k % (4 / G)) * stg_run(G, CR);
-    for (int i = lane; i < DS; i += 32) p[i] = 0.f;
-    for (int i = lane; i < DS + 8; i += 32) p[(G + CR) * DS + i] = 0.f;
-  }
-}
-
-// ---- add the warps' lag sums of a tile to V, in a fixed order: thread per (kappa, lambda).
-// Under the real part (kappa, lambda) and the conjugate of (-kappa, -lambda) are the same, so V
-// keeps lambda >= 0 only and takes both. v: planes re hi, re lo, im hi, im lo of nv floats.
-template <int G, int CR>
-__device__ __forceinline__ void corr_combine(const JobRegs& J, int row0, int col0, int cols,
-                                             const float* sl, float* v, int nv, int tid) {
-  constexpr int NU = 8 * (G + CR), SF = slice_floats(G, CR);
-  constexpr int RW = 8 * G, CW = 8 * CR;               // slots of a row run and of a column run
-  const int ny = J.ny, mx = J.mx, nyp = J.nyp;
-  const int a0 = row0 / nyp, a1 = min((row0 + 127) / nyp, J.nx - 1);         // E-W rows of the rows
-  const int b0 = col0 / nyp, b1 = min((col0 + cols - 1) / nyp, J.nx - 1);   // and of the columns
-  const int dlo = a0 - b1, dhi = a1 - b0;              // separations ia - ib in the tile
-  int r0 = dlo % mx;
-  if (r0 < 0) r0 += mx;
-  const int cand = nyp > CW ? 2 : 1;                   // column runs that can hold a lag
-  // 2^lg threads per E-W class, one lambda each
-  const int lg = min(8, 32 - __clz(ny - 1 | 15)), kstep = EPI >> lg;
-  for (int lam0 = tid & ((1 << lg) - 1); lam0 < ny; lam0 += 1 << lg) {
-#pragma unroll 1
-    for (int kap0 = tid >> lg; kap0 < mx; kap0 += kstep) {
-      Cdd s = dd_zero();
-      bool any = false;
-#pragma unroll 1
-      for (int mir = 0; mir < (lam0 ? 2 : 1); ++mir) {
-        const int lam = mir ? -lam0 : lam0;
-        int d = (mir && kap0 ? mx - kap0 : kap0) - r0;
-        d = dlo + (d < 0 ? d + mx : d);                // first separation of class kappa
-#pragma unroll 1
-        for (; d <= dhi; d += mx) {
-          const int ie = min(a1, b1 + d);
-#pragma unroll 1
-          for (int ia = max(a0, b0 + d); ia <= ie; ++ia) {
-            const int base = (ia - d) * nyp - col0;    // tile column of slot 0 of row ib, may be negative
-            const int ylo = max(0, -base), yhi = min(nyp, cols - base);
-            const int ra = ia * nyp - row0;            // CTA row of slot (ia, 0), may be negative
-            const int rend = min(ra + nyp, 128);
-            any = true;
-#pragma unroll 1
-            for (int row = max(ra, 0); row < rend; row += RW) {
-              const int t = row - ra - lam;            // = lag + yb, lag = b - a in -(RW-1) .. CW-1
-              const int lim = min(yhi, t + RW);
-              int yb = (max(t - (CW - 1), ylo) + CW - 1) & ~(CW - 1);
-              const int rs = row / RW;
-              const float* p = sl + ((rs * G) >> 2) * (2 * SF) + (rs & (4 / G - 1)) * (16 / CR) * NU + t + RW - 1;
-#pragma unroll 1
-              for (int e = 0; e < cand; ++e, yb += CW) {
-                const int run = (base + yb) / CW;
-                const float* q = p + (run / (16 / CR)) * (8 * SF) + (run & (16 / CR - 1)) * NU - yb;
-                if (yb < lim) dd_acc(s, make_float2(q[0], mir ? -q[SF] : q[SF]));
-              }
-            }
-          }
-        }
-      }
-      if (any) {
-        const int o = kap0 * ny + lam0;
-        const Cdd w = dd_add(Cdd{make_float2(v[o], v[2 * nv + o]), make_float2(v[nv + o], v[3 * nv + o])}, s);
-        v[o] = w.h.x;
-        v[nv + o] = w.l.x;
-        v[2 * nv + o] = w.h.y;
-        v[3 * nv + o] = w.l.y;
-      }
-    }
-  }
-}
-
-// The same where a tile lies in one pair of E-W rows (nyp a multiple of 256): thread per lambda.
-// Lag l of the CTA's 128 x cols tile is, for row run rs, in column run (l + 32 rs) / (8 CR) and in
-// the next one.
-template <int CR>
-__device__ __forceinline__ void corr_combine_one(const JobRegs& J, int row0, int col0, int cols,
-                                                 const float* sl, float* v, int nv, int tid) {
-  constexpr int CW = 8 * CR, NU = CW + 32, SF = slice_floats(4, CR), RPW = 16 / CR;
-  const int ny = J.ny, ia = row0 / J.nyp, ib = col0 / J.nyp;
-  int kap = (ia - ib) % J.mx;
-  if (kap < 0) kap += J.mx;
-  const int D = (row0 - ia * J.nyp) - (col0 - ib * J.nyp), nr = cols / CW;   // lambda = D - l
-  for (int o = tid; o < ny; o += EPI) {
-#pragma unroll 1
-    for (int mir = 0; mir < (o ? 2 : 1); ++mir) {
-      const int l = mir ? D + o : D - o;
-      if (l < -127 || l >= cols) continue;
-      Cdd s = dd_zero();
-#pragma unroll
-      for (int rs = 0; rs < 4; ++rs) {
-        const int x = l + 32 * rs + 128, run = x / CW - 128 / CW, w = x & (CW - 1);   // x > 0
-        const float* p = sl + rs * (2 * SF);
-        float2 a = make_float2(0.f, 0.f), b = a;
-        if (run >= 0 && run < nr) {
-          const float* q = p + (run / RPW) * (8 * SF) + (run & (RPW - 1)) * NU + w + 31;
-          a = make_float2(q[0], q[SF]);
-        }
-        if (w >= CW - 31 && run + 1 >= 0 && run + 1 < nr) {
-          const float* q = p + ((run + 1) / RPW) * (8 * SF) + ((run + 1) & (RPW - 1)) * NU + w + 31 - CW;
-          b = make_float2(q[0], q[SF]);
-        }
-        dd_acc(s, a);
-        dd_acc(s, b);
-      }
-      if (mir) {
-        s.h.y = -s.h.y;
-        s.l.y = -s.l.y;
-      }
-      const int kp = mir && kap ? J.mx - kap : kap, e = kp * ny + o;
-      const Cdd w = dd_add(Cdd{make_float2(v[e], v[2 * nv + e]), make_float2(v[nv + e], v[3 * nv + e])}, s);
-      v[e] = w.h.x;
-      v[nv + e] = w.l.x;
-      v[2 * nv + e] = w.h.y;
-      v[3 * nv + e] = w.l.y;
-    }
-  }
-}
-
+// The same as a function of its own, whose registers do not add to the other splits': inlined, the four
+// splits of complex weights and the four of real ones beside them in a launch spill inside the loops
+// (8x64 with gains 1363 us, with calls 1227).
 template <int G, int CR, bool CPLX>
-__device__ __forceinline__ void corr_half(uint32_t tacc, int half, int warp, int lane, int cols,
-                                          int row0, int col0, float scale, bool diag, uint32_t drained,
-                                          uint32_t drained2, const float* ws, int wslots, float* stg, float* sl) {
-  // real weights: the real half is one component of V, the imaginary half the other
-  corr_phase<G, CR, CPLX>(tacc, warp & 3, warp >> 2, cols, row0, col0, scale, ws, wslots,
-                          stg + warp * (CPLX ? 2 : 1) * stg_floats(G, CR),
-                          sl + (warp * 2 + half) * slice_floats(G, CR), diag, drained, drained2, lane);
-}
-
-// The same where a row of slots divides the CTA's 128 rows (NYP = 16, 32, 64 or 128): the pairs of
-// E-W rows are whole blocks, NYP / (8G) x NYP / (8CR) run pairs each, and everything but the class
-// is known at compile time.
-template <int G, int CR, int NYP>
-__device__ __forceinline__ void corr_combine_blocks(const JobRegs& J, int row0, int col0, int cols,
-                                                    const float* sl, float* v, int nv, int tid) {
-  constexpr int NU = 8 * (G + CR), SF = slice_floats(G, CR);
-  constexpr int RW = 8 * G, CW = 8 * CR, NR = NYP / RW, NC = NYP / CW, NA = 128 / NYP;
-  const int ny = J.ny, mx = J.mx, nb = cols / NYP;
-  int r0 = (row0 / NYP - col0 / NYP) % mx;             // first row minus first column, mod mx
-  if (r0 < 0) r0 += mx;
-  const int lg = min(8, 32 - __clz(ny - 1 | 15)), kstep = EPI >> lg;
-  const int lam0 = tid & ((1 << lg) - 1);              // ny <= NYP <= 128: one lambda per thread
-  if (lam0 >= ny) return;
-#pragma unroll 1
-  for (int kap0 = tid >> lg; kap0 < mx; kap0 += kstep) {
-    Cdd s = dd_zero();
-#pragma unroll 1
-    for (int mir = 0; mir < (lam0 ? 2 : 1); ++mir) {
-      const int lam = mir ? -lam0 : lam0;
-      int b = r0 + (mir ? kap0 : -kap0);               // column row of class kappa for the first row
-      b += b < 0 ? mx : b >= mx ? -mx : 0;
-#pragma unroll
-      for (int al = 0; al < NA; ++al) {
-        for (int be = b; be < nb; be += mx) {
-#pragma unroll
-          for (int rr = 0; rr < NR; ++rr)
-#pragma unroll
-            for (int c = 0; c < NC; ++c) {
-              const int rs = al * NR + rr, run = be * NC + c, lag = rr * RW - c * CW - lam;
-              const float* q = sl + ((rs * G) >> 2) * (2 * SF) + (rs & (4 / G - 1)) * (16 / CR) * NU +
-                               (run / (16 / CR)) * (8 * SF) + (run & (16 / CR - 1)) * NU + lag + RW - 1;
-              if (lag > -RW && lag < CW) dd_acc(s, make_float2(q[0], mir ? -q[SF] : q[SF]));
-            }
-        }
-        if (++b == mx) b = 0;
-      }
-    }
-    const int o = kap0 * ny + lam0;
-    const Cdd w = dd_add(Cdd{make_float2(v[o], v[2 * nv + o]), make_float2(v[nv + o], v[3 * nv + o])}, s);
-    v[o] = w.h.x;
-    v[nv + o] = w.l.x;
-    v[2 * nv + o] = w.h.y;
-    v[3 * nv + o] = w.l.y;
-  }
+__device__ __noinline__ void corr_phase_call(uint32_t tacc, int cols, int row0, int col0, float scale,
+                                             int ws0, int wslots, int stg0, int v0, int nv, int half,
+                                             int nx, int ny, int nyp, int mx, float lscale,
+                                             bool diag, uint32_t drained, uint32_t drained2) {
+  corr_phase<G, CR, CPLX>(tacc, cols, row0, col0, scale, ws0, wslots, stg0, v0, nv, half, nx, ny, nyp,
+                          mx, lscale, diag, drained, drained2);
 }
 
 // Entries of a twiddle table that a transform of n reads: half of them where n is a power of two.
@@ -764,8 +678,8 @@ __device__ void corr_beams(const CorrJob& J, int64_t item, int rank, float* v, i
       y = s.h;
     }
     // intensities are sums of squares: rounding may leave a beam without power just below 0
-    dst[A0 * my + B] = y.x < 0.f ? 0.f : y.x;
-    if (A0 + 1 < mx) dst[(A0 + 1) * my + B] = y.y < 0.f ? 0.f : y.y;
+    dst[A0 * my + B] = y.x < 0.f ? 0.f : ldexpf(y.x, J.out_exp);
+    if (A0 + 1 < mx) dst[(A0 + 1) * my + B] = y.y < 0.f ? 0.f : ldexpf(y.y, J.out_exp);
   }
 }
 
@@ -971,10 +885,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(corr::NT, 1)
     abort_flag = 0;
   }
   {
-    float* v = reinterpret_cast<float*>(smem + Y.v);
-    for (int i = tid; i < 4 * P.s.vlen; i += NT) v[i] = 0.f;
-    float* stg = reinterpret_cast<float*>(smem + Y.stg);
-    for (int i = tid; i < 8 * P.s.stg; i += NT) stg[i] = 0.f;
+    int* v = reinterpret_cast<int*>(smem + Y.v);
+    for (int i = tid; i < 4 * P.s.vlen; i += NT) v[i] = 0;
   }
   tc::fence_before_sync();
   cluster_sync();
@@ -993,28 +905,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(corr::NT, 1)
   if (warp < 8) {
     // ================================================= epilogue
     float* ws = reinterpret_cast<float*>(smem + Y.w);
-    float* vv = reinterpret_cast<float*>(smem + Y.v);
+    int* vv = reinterpret_cast<int*>(smem + Y.v);
     float* stg = reinterpret_cast<float*>(smem + Y.stg);
-    float* sl = reinterpret_cast<float*>(smem + Y.sl);
     float4* tab = reinterpret_cast<float4*>(smem + Y.tab);
     const int wslots = P.s.wslots;
     const uint32_t rf = map_rank(tc::smem_u32(bars + RF), 0), imf = map_rank(tc::smem_u32(bars + IF), 0);
     const CorrJob* last = nullptr;
-    auto zero_rows = [&]() {                           // for the split of the job `last`
-      const int c = CPLX && !last->a.real_w ? 2 : 1;
-      switch (last->mode) {
-        case 0: corr_zero_rows<4, 8>(stg + warp * c * stg_floats(4, 8), c, lane); break;
-        case 1: corr_zero_rows<4, 4>(stg + warp * c * stg_floats(4, 4), c, lane); break;
-        default: corr_zero_rows<2, 2>(stg + warp * c * stg_floats(2, 2), c, lane); break;
-      }
-    };
     int64_t item = pair;
     int job = 0;
     uint32_t ph = 0, iph = 0;                          // tile and item parities
     bool ok = true;
     while (item < P.total && ok) {
       const CorrJob& J = find_job(P, item, job);
-      const JobRegs R{J.a.nx, J.ny, J.nyp, J.np, J.nt, J.a.mx, J.mode + (CPLX && !J.a.real_w ? 4 : 0)};
+      const JobRegs R{J.a.nx, J.ny, J.nyp, J.np, J.nt, J.a.mx, J.mode + (CPLX && !J.a.real_w ? 4 : 0),
+                      J.rscale, J.lscale};
       const int nv = R.mx * R.ny;
       if (&J != last) {                                // weights in slot order, zeros between
         bar_epi();
@@ -1022,27 +926,33 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(corr::NT, 1)
           const int ix = s / J.nyp, iy = s - ix * J.nyp;
           float2 w = make_float2(0.f, 0.f);
           if (ix < J.a.nx && iy < J.ny) w = J.a.w[ix * J.ny + iy];
-          ws[s] = w.x;
-          if (CPLX) ws[wslots + s] = w.y;
+          ws[s] = ldexpf(w.x, J.w_exp);
+          if (CPLX) ws[wslots + s] = ldexpf(w.y, J.w_exp);
         }
         const int ty = tw_len(J.a.my), tx = tw_len(J.a.mx);
         for (int i = tid; i < ty + tx; i += EPI) tab[i] = J.a.cw[i < ty ? i : J.a.my + i - ty];
         last = &J;
-        zero_rows();
         bar_epi();
       }
       for (int I = 0; I < R.nt && ok; ++I)
         for (int Jc = I; Jc < R.nt && ok; ++Jc) {
           const int cols = tile_cols(R.np, Jc);
           const int row0 = 256 * I + 128 * (int)rank, col0 = 256 * Jc;
-          // each e4m3 operand carries 2^-9; off the diagonal a tile stands for its mirror too
-          const float s18 = 262144.f;
+          // off the diagonal a tile stands for its mirror too
           if (CPLX && (R.mode & 4)) {                  // complex weights: both halves at once
             ok = wait_warp(RD, ph) && wait_warp(ID, ph);
             if (ok) {
               tc::fence_after_sync();
-              if (R.mode == 5) corr_half<4, 4, CPLX>(tbase, 0, warp, lane, cols, row0, col0, 2.f * s18, I == Jc, rf, imf, ws, wslots, stg, sl);
-              else corr_half<2, 2, CPLX>(tbase, 0, warp, lane, cols, row0, col0, 2.f * s18, I == Jc, rf, imf, ws, wslots, stg, sl);
+#define FFTBF_PHASE(F, G, CR)                                                                           \
+  F<G, CR, CPLX>(tbase, cols, row0, col0, 2.f * R.rscale, Y.w, wslots, Y.stg, Y.v, nv, 0, R.nx, R.ny,    \
+                 R.nyp, R.mx, R.lscale, I == Jc, rf, imf)
+              switch (R.mode & 3) {
+                case 3: FFTBF_PHASE(corr_phase_call, 4, 16); break;
+                case 0: FFTBF_PHASE(corr_phase_call, 4, 8); break;
+                case 1: FFTBF_PHASE(corr_phase_call, 4, 4); break;
+                default: FFTBF_PHASE(corr_phase, 2, 2); break;
+              }
+#undef FFTBF_PHASE
             }
           } else {
 #pragma unroll 1
@@ -1050,41 +960,26 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(corr::NT, 1)
               ok = wait_warp(half ? ID : RD, ph);
               if (!ok) break;
               tc::fence_after_sync();
-              const float scale = (half == 0 && I == Jc) ? s18 : 2.f * s18;
-              const uint32_t tacc = tbase + 256 * half;
+#define FFTBF_PHASE(F, G, CR)                                                                         \
+  F<G, CR, false>(tbase + 256 * half, cols, row0, col0, half == 0 && I == Jc ? R.rscale : 2.f * R.rscale, \
+                  Y.w, 0, Y.stg, Y.v, nv, half, R.nx, R.ny, R.nyp, R.mx, R.lscale, false,                 \
+                  half ? imf : rf, 0)
+#define FFTBF_REAL(G, CR)                                                                             \
+  if constexpr (CPLX) FFTBF_PHASE(corr_phase_call, G, CR);                                              \
+  else FFTBF_PHASE(corr_phase, G, CR)
               switch (R.mode) {
-                case 0: corr_half<4, 8, false>(tacc, half, warp, lane, cols, row0, col0, scale, false, half ? imf : rf, 0, ws, wslots, stg, sl); break;
-                case 1: corr_half<4, 4, false>(tacc, half, warp, lane, cols, row0, col0, scale, false, half ? imf : rf, 0, ws, wslots, stg, sl); break;
-                default: corr_half<2, 2, false>(tacc, half, warp, lane, cols, row0, col0, scale, false, half ? imf : rf, 0, ws, wslots, stg, sl); break;
+                case 3: FFTBF_REAL(4, 16); break;
+                case 0: FFTBF_REAL(4, 8); break;
+                case 1: FFTBF_REAL(4, 4); break;
+                default: FFTBF_REAL(2, 2); break;
               }
+#undef FFTBF_REAL
+#undef FFTBF_PHASE
             }
           }
-          ok = bar_epi_all(ok);                        // the warps leave together or not at all
-          if (!ok) break;
-#define FFTBF_COMBINE(F) F(R, row0, col0, cols, sl, vv, nv, tid)
-          switch (R.mode & 3) {
-            case 0:
-              if ((R.nyp & 255) == 0) FFTBF_COMBINE(corr_combine_one<8>);
-              else if (R.nyp == 128) FFTBF_COMBINE((corr_combine_blocks<4, 8, 128>));
-              else if (R.nyp == 64) FFTBF_COMBINE((corr_combine_blocks<4, 8, 64>));
-              else FFTBF_COMBINE((corr_combine<4, 8>));
-              break;
-            case 1:
-              if ((R.nyp & 255) == 0) FFTBF_COMBINE(corr_combine_one<4>);
-              else if (CPLX && R.nyp == 128) FFTBF_COMBINE((corr_combine_blocks<4, 4, 128>));
-              else if (CPLX && R.nyp == 64) FFTBF_COMBINE((corr_combine_blocks<4, 4, 64>));
-              else if (R.nyp == 32) FFTBF_COMBINE((corr_combine_blocks<4, 4, 32>));
-              else FFTBF_COMBINE((corr_combine<4, 4>));
-              break;
-            default:
-              if (R.nyp == 16) FFTBF_COMBINE((corr_combine_blocks<2, 2, 16>));
-              else FFTBF_COMBINE((corr_combine<2, 2>));
-              break;
-          }
-#undef FFTBF_COMBINE
-          bar_epi();
           ph ^= 1;
         }
+      ok = bar_epi_all(ok);                            // the warps leave together or not at all
       if (!ok) break;
       // ---- item complete: each CTA adds the other's part of V to its own and transforms its share
       // of the beams; V is cleared once the other has read it. One thread releases and acquires
@@ -1100,21 +995,27 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(corr::NT, 1)
       float* u = stg;                                  // the sum, then the transform's buffer after it
 #pragma unroll 1
       for (int i0 = tid; i0 < nv; i0 += 4 * EPI) {
-        float4 p[4];
+        int p[4][4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           const int i = min(i0 + k * EPI, nv - 1);
-          asm volatile("ld.shared::cluster.f32 %0, [%1];\n" : "=f"(p[k].x) : "r"(peer + 4 * i) : "memory");
-          asm volatile("ld.shared::cluster.f32 %0, [%1];\n" : "=f"(p[k].y) : "r"(peer + 4 * (nv + i)) : "memory");
-          asm volatile("ld.shared::cluster.f32 %0, [%1];\n" : "=f"(p[k].z) : "r"(peer + 4 * (2 * nv + i)) : "memory");
-          asm volatile("ld.shared::cluster.f32 %0, [%1];\n" : "=f"(p[k].w) : "r"(peer + 4 * (3 * nv + i)) : "memory");
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            asm volatile("ld.shared::cluster.b32 %0, [%1];\n" : "=r"(p[k][c]) : "r"(peer + 4 * (c * nv + i)) : "memory");
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           const int i = i0 + k * EPI;
           if (i >= nv) break;
-          const Cdd x{make_float2(vv[i], vv[2 * nv + i]), make_float2(vv[nv + i], vv[3 * nv + i])};
-          const Cdd t = dd_add(x, Cdd{make_float2(p[k].x, p[k].z), make_float2(p[k].y, p[k].w)});
+          // whole numbers and 2^-19 units, each to a float and its remainder
+          const int re = vv[i] + p[k][0], rl = vv[nv + i] + p[k][1];
+          const int im = vv[2 * nv + i] + p[k][2], il = vv[3 * nv + i] + p[k][3];
+          auto two = [](int x, int y, float s) {
+            const float fx = (float)x, fy = (float)y;
+            return Cdd{make_float2(s * fx, s * fy),
+                       make_float2(s * (float)(x - (int)fx), s * (float)(y - (int)fy))};
+          };
+          const Cdd t = dd_add(two(re, im, 1.f), two(rl, il, 1.f / R.lscale));
           u[i] = t.h.x;
           u[nv + i] = t.l.x;
           u[2 * nv + i] = t.h.y;
@@ -1130,8 +1031,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(corr::NT, 1)
       }
       ok = bar_epi_all(ok);
       if (!ok) break;
-      for (int i = tid; i < 4 * nv; i += EPI) vv[i] = 0.f;
-      zero_rows();
+      for (int i = tid; i < 4 * nv; i += EPI) vv[i] = 0;
       bar_epi();
       iph ^= 1;
       item += npairs;
@@ -1209,17 +1109,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(corr::NT, 1)
 
 // ------------------------------------------------------------------------- host side --
 // Split of a lattice into slots: nyp and the (G, CR) of the epilogue.
-static void corr_split(int ny, bool cplx, int* nyp, int* mode) {
+static void corr_split(int ny, int* nyp, int* mode) {
   auto up = [&](int m) { return (ny + m - 1) / m * m; };
   // multiples of 16 stay as they are (slots = feeds, staged by TMA); others are rounded up, to
   // the longer runs where the padding is small
   if (ny % 16 == 0) *nyp = ny;
   else *nyp = up(ny >= 192 ? 64 : ny >= 96 ? 32 : 16);
-  // the longest column runs that divide a row: 64, 32 or 16 slots (32 at most with complex
-  // weights, whose two components double the staging). Runs of 128 shorten the gather a little
-  // but cost a stage of operands: 4x256 5.13 ms against 5.0 (4096 windows x channels).
+  // the longest column runs that divide a row: 128, 64, 32 or 16 slots (a run of n 8-slot groups has
+  // n / 4 + 1 gathers; 4x256, 1024 work items: 1614 us at 128 slots, 1720 at 64)
   const int n = *nyp;
-  *mode = n % 64 == 0 && !cplx ? 0 : n % 32 == 0 ? 1 : 2;
+  *mode = n % 128 == 0 ? 3 : n % 64 == 0 ? 0 : n % 32 == 0 ? 1 : 2;
 }
 
 bool corr_make_job(const BeamArgs& a, CorrJob* J) {
@@ -1227,16 +1126,30 @@ bool corr_make_job(const BeamArgs& a, CorrJob* J) {
   j.a = a;
   j.ny = a.ny;
   j.nant = a.nx * a.ny;
-  corr_split(a.ny, !a.real_w, &j.nyp, &j.mode);
+  corr_split(a.ny, &j.nyp, &j.mode);
   j.np = a.nx * j.nyp;
   j.nt = (j.np + 255) / 256;
   const int64_t nsnap = (int64_t)a.n_int * a.npol;
   j.nch = (int)((nsnap + corr::KS - 1) / corr::KS);
   j.tma = (a.ny & 15) == 0 && (reinterpret_cast<uintptr_t>(a.volts) & 15) == 0 && KS % a.npol == 0;
   j.nitems = a.nwin * a.nfreq;
+  // Units of V. With weights below 2 (w_exp) a product with its mirror is below 2 128 4 2^ns; a unit
+  // is 2^-19 of that, and with n = nx ny ceil(nx / mx) feed pairs of one separation above 1024 2^e
+  // times it (n <= 1024 2^e): V stays below 2^30 units. What lies below a unit, at most 1/2 + 2^-5 a
+  // product and twice that with complex weights, sums to 1.1 2^(11 + e) units at most, and is kept in
+  // 2^-(19 - e) of one: below 2^31. With e = 4 that is 2^-30 of the largest product, rounded once for
+  // every 16 or more of them; lattices folded further take the transform.
+  auto clog2 = [](int64_t n) { int l = 0; while (((int64_t)1 << l) < n) ++l; return l; };
+  const int ns = clog2(nsnap), e = std::max(0, clog2((int64_t)j.nant * ((a.nx + a.mx - 1) / a.mx)) - 10);
+  const int z = a.real_w ? 0 : 31 - ns, w = a.w_exp == kNoExp ? 0 : a.w_exp;
+  j.w_exp = z - w;                                     // complex: z = w_b^* R up to 2^21
+  j.rscale = ldexpf(1.f, 27 - ns - e - 2 * z);         // R carries 2^-18
+  j.lscale = ldexpf(1.f, 19 - e);
+  j.out_exp = ns - 9 + e + 2 * w;
   *J = j;
   // sums stay exact to 128 * 2^16 snapshots with room; V and the transform fit beside the ring
-  return a.cw && j.np <= 2048 && nsnap <= 65536 && (int64_t)a.mx * a.ny <= corr::VMAX &&
+  return a.cw && a.w_exp != kNoExp && e <= 4 && j.np <= 2048 && nsnap <= 65536 &&
+         (int64_t)a.mx * a.ny <= corr::VMAX &&
          (int64_t)((a.mx + 1) / 2) * a.my <= 2048;
 }
 
@@ -1251,11 +1164,10 @@ bool corr_sizes(const CorrJob* jobs, int n, CorrSizes* out) {
   for (int i = 0; i < n; ++i) {
     const CorrJob& j = jobs[i];
     const int m = j.mode, c = j.a.real_w ? 1 : 2;
-    const int G = m == 2 ? 2 : 4, CR = m == 0 ? 8 : m == 1 ? 4 : 2;
+    const int G = m == 2 ? 2 : 4, CR = m == 3 ? 16 : m == 0 ? 8 : m == 1 ? 4 : 2;
     s.wslots = std::max(s.wslots, 256 * j.nt);
     s.vlen = std::max(s.vlen, j.a.mx * j.ny);
-    s.stg = std::max({s.stg, c * stg_floats(G, CR), (4 * j.a.mx * j.ny + ((j.a.mx + 1) / 2 + 1) / 2 * j.a.my * 4 + 7) / 8});
-    s.slice = std::max(s.slice, 2 * slice_floats(G, CR));
+    s.stg = std::max({s.stg, stg_floats(G, CR, c), (4 * j.a.mx * j.ny + ((j.a.mx + 1) / 2 + 1) / 2 * j.a.my * 4 + 7) / 8});
     s.tab = std::max(s.tab, tw_len(j.a.my) + tw_len(j.a.mx));
   }
   s.stg = (s.stg + 3) & ~3;
@@ -1316,17 +1228,18 @@ int corr_launch(CorrParams& p, int nsm, cudaStream_t st) {
 }
 
 // Where the covariance beats the transform of every snapshot. Both are taken as microseconds of 608
-// work items (eight per CTA pair), measured on a GB300 from 8 to 512 snapshots per window:
-//   covariance  34 us per tile and 55 us per item, 1.4 times that with complex weights (epilogue
-//               and transform of V, whatever the window; 4x256: 398 us, 8x64 160, 16x16 107),
-//               and from there 0.021 us per snapshot and MMA unit (a 256 x 256 product of the
-//               chunk: 3 a diagonal tile, 4 another; 4x256 772 us at 768 snapshots), three
-//               times that where the voltages cannot come by TMA;
-//   transform   us per snapshot and 1000 beams: 0.8 the 512-beam kernels (4x256: 827 us at 512),
-//               0.6 the 32-beam kernel, 1.1 those of 1024 and 2048 beams, 1.9 the other FFT
-//               kernels (8x64: 980 us at 512); the direct DFT 1.0 for every N-S feed. The
-//               split-FP16 kernel (split) 1.3 (4x256: 2060 us at 768).
-// So 4x256 changes over near 300 snapshots, 8x64 near 90, 16x16 near 400. Only the plan's sizes
+// work items (eight per CTA pair), measured on a GB300 from 16 to 768 snapshots per window:
+//   covariance  per tile, whatever the window (the epilogue), 41 us for rows of 128 slots, 50 of 64 or
+//               32 and 105 of 16, with complex weights 82 and 108; per item 40 us and 0.043 per value
+//               of a CTA's transform (4x256: 470 us, 8x64 205, 16x16 152; complex 874, 298, 163). The
+//               products run under that in part, 0.0182 us per snapshot and MMA unit (a 256 x 256
+//               product of the chunk: 3 a diagonal tile, 4 another; 4x256 914 us at 768 snapshots).
+//               Where the voltages cannot come by TMA 0.25 us per snapshot and tile (4x100: 616 us);
+//   transform   us per snapshot and 1000 beams: 0.8 the 512-beam kernels (4x256: 826 us at 512),
+//               0.58 the 32-beam kernel, 1.2 the 256-beam ones, 1.1 those of 1024 and 2048 beams, 1.9
+//               the other FFT kernels (8x64: 979 us at 512); the direct DFT 1.0 for every N-S feed.
+//               The split-FP16 kernel (split) 1.3 (4x256: 2060 us at 768).
+// So 4x256 changes over near 420 snapshots, 8x64 near 110, 16x16 near 600. Only the plan's sizes
 // enter, never the number of windows or the pointer: a window's beams do not depend on its call.
 bool corr_preferred(const BeamArgs& a, bool split) {
   CorrJob j;
@@ -1341,12 +1254,15 @@ bool corr_preferred(const BeamArgs& a, bool split) {
     tiles += c + 1;
     units += w * (3 + 4 * c);
   }
-  const double fixed = (34.0 * tiles + 55.0) * (a.real_w ? 1.0 : 1.4);
-  const double cov = std::max(fixed, 0.6 * fixed + 0.021 * (j.ny % 16 == 0 && corr::KS % a.npol == 0 ? 1 : 3) * units * nsnap);
+  static const double kTile[4] = {50.0, 50.0, 105.0, 41.0}, kTileC[4] = {82.0, 82.0, 108.0, 82.0};
+  const double fixed = tiles * (a.real_w ? kTile : kTileC)[j.mode] + 40.0 + 0.043 * a.my * (((a.mx + 1) / 2 + 1) / 2);
+  const double cov = j.ny % 16 == 0 && corr::KS % a.npol == 0
+                         ? std::max(fixed, (a.real_w ? 0.85 : 1.0) * fixed + 0.0182 * units * nsnap)
+                         : std::max(fixed, (a.real_w ? 17.0 * tiles : 0.5 * fixed) + 0.25 * tiles * nsnap);
   double per;                                          // us per snapshot
   if (split) per = 1.3e-3 * nout;
   else if (fp32_n512_supported(a)) per = 0.8e-3 * nout;
-  else if (fp32_warp_supported(a)) per = (a.my == 32 ? 0.6e-3 : a.my >= 1024 ? 1.1e-3 : 1.9e-3) * nout;
+  else if (fp32_warp_supported(a)) per = (a.my == 32 ? 0.58e-3 : a.my == 256 ? 1.2e-3 : a.my >= 1024 ? 1.1e-3 : 1.9e-3) * nout;
   else if (fp32_fft_supported(a.mx, a.my)) per = 1.9e-3 * std::max<double>(nout, j.nant);
   else per = 1e-3 * nout * a.nyf;
   return cov < per * nsnap;

@@ -13,14 +13,18 @@ struct CorrJob {
   BeamArgs a;
   int ny, nyp;          // N-S feeds, and their slots (a multiple of 16, 32 or 64)
   int nant, np, nt;     // feeds, slots, tiles of 256 slots per axis
-  int nch;              // chunks of 32 snapshots per window
-  int mode;             // epilogue split 0..2: 8-slot groups per run 4x8, 4x4, 2x2
+  int nch;              // stages of kCorrSteps snapshots per window
+  int mode;             // epilogue split 0..3: 8-slot groups per run 4x8, 4x4, 2x2, 4x16
   int tma;              // voltages staged by TMA
+  int w_exp;            // the weights are held times 2^w_exp
+  float rscale;         // and those of the rows times this, for sums in units of V
+  float lscale;         // what lies below a unit is kept times this
+  int out_exp;          // beams are V's transform times 2^out_exp
   int64_t item0, nitems;
 };
 struct CorrSizes {      // shared-memory sizes, the largest over the launch's jobs
   int ns, nr;           // operand stages, staged voltage tiles
-  int wslots, vlen, stg, slice, tab;
+  int wslots, vlen, stg, tab;
   int cplx;             // some weights are complex
   int tma;              // every job's voltages are staged by TMA
 };

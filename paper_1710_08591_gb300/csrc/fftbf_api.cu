@@ -53,6 +53,16 @@ static void remember_stream(fftbf_plan* p, cudaStream_t st) {
     p->streams_used.push_back(st);
 }
 
+int weight_exp(const float* w, int64_t n) {
+  double m = 0.0;                                      // |w|^2: within FP64 for any FP32 weights
+  for (int64_t i = 0; i < n; ++i) {
+    const double re = w[2 * i], im = w[2 * i + 1], a = re * re + im * im;
+    if (!std::isfinite(a)) return kNoExp;
+    m = std::max(m, a);
+  }
+  return m > 0.0 ? (int)std::floor(0.5 * std::ilogb(m)) : 0;
+}
+
 class DeviceGuard {
  public:
   explicit DeviceGuard(int dev) {
@@ -108,6 +118,7 @@ fftbf_plan* fftbf_plan_create(int nx, int ny, int pad_x, int pad_y, int npol, in
     }
     p->real_w = true;
     for (int i = 0; i < nant; ++i) p->real_w = p->real_w && p->h_w[2 * i + 1] == 0.f;
+    p->w_exp = weight_exp(p->h_w.data(), nant);
     e = cudaMemcpy(p->d_w, p->h_w.data(), sizeof(float2) * nant, cudaMemcpyHostToDevice);
   }
   // the table of the covariance route, for plans that take it in some precision (a rule on sizes);
@@ -118,6 +129,7 @@ fftbf_plan* fftbf_plan_create(int nx, int ny, int pad_x, int pad_y, int npol, in
     a.npol = npol; a.nfreq = nfreq; a.n_int = n_int;
     a.nyf = std::min(ny, pad_y);
     a.real_w = p->real_w ? 1 : 0;
+    a.w_exp = p->w_exp;
     float4 here;
     a.cw = &here;
     if (corr_preferred(a) || (tc_supported(nx, ny, pad_x, pad_y) && corr_preferred(a, true)))
@@ -219,6 +231,7 @@ int fftbf_execute(fftbf_plan* p, const uint8_t* volts, int64_t T, float* beams, 
   a.real_w = p->real_w ? 1 : 0;
   a.cw = p->d_cw;
   a.err = p->d_err;
+  a.w_exp = p->w_exp;
   const int nsnap = p->n_int * p->npol;
   int S = kMaxElems / (p->mx * p->my);
   if (S < 1) S = 1;

@@ -57,7 +57,12 @@ struct BeamArgs {
   int64_t nwin;           // windows in this call
   const float4* cw;       // two-float exp(-2 pi i k / my), k < my, then exp(-2 pi i k / mx): (cos hi, lo, -sin hi, lo)
   int* err;               // device error word of bounded waits; null: no kernel that needs one
+  int w_exp;              // weight_exp of the weights (covariance form)
 };
+// Exponent of the largest |w| of n weights (re, im interleaved): |w| < 2^(w_exp + 1); 0 if all are
+// zero, kNoExp if one is not finite.
+constexpr int kNoExp = INT32_MIN;
+int weight_exp(const float* w, int64_t n);
 
 // Launch the FP32 fused beam kernel. Returns FFTBF_OK or an error code.
 int launch_beams_fp32(const BeamArgs& a, int nsm, cudaStream_t st);
@@ -209,6 +214,7 @@ struct fftbf_plan {
   fftbf::HostPipe pipe;
   std::vector<float> h_w;         // host copy of the weights (re, im interleaved)
   bool real_w = false;            // every weight has a zero imaginary part
+  int w_exp = 0;                  // exponent of the largest weight (weight_exp)
   uint16_t* d_b1 = nullptr;       // tensor-core stage matrices for the selected precision
   uint16_t* d_b2 = nullptr;
   uint16_t* d_b1lo = nullptr;     // split FP16 form: residuals of the stage matrices

@@ -225,3 +225,88 @@ def test_server_ticks_reuse_slots_for_other_lattices():
                 assert np.array_equal(o, want.cpu().numpy()[0])
     for p in plans:
         p.close()
+
+
+STRONG = [(1.5, 2.5), (5.0, 1.0), (6.0, 1.0), (6.5, 0.5), (7.0, 0.3)]    # source amplitude, noise sigma
+
+
+@pytest.mark.parametrize("weights", ["half_sine", "random"])
+@pytest.mark.parametrize("shape", [(4, 256, 4, 512, 2, 384), (8, 64, 8, 128, 2, 256), (4, 32, 4, 64, 2, 256),
+                                   (16, 16, 16, 32, 2, 256), (3, 37, 5, 73, 1, 200)],
+                         ids=lambda s: "x".join(map(str, s[:4])))
+def test_weak_beams_beside_a_strong_source(shape, weights, monkeypatch):
+    """Every beam within 1e-6, tighter than TOL_BEAM and than what the transform of every snapshot
+    reaches on the larger lattices: the sums keep 2^-37 of a source's power or better and the beams
+    here are down to 2^-19 of it, so little more than the last rounding (2^-24) is left."""
+    nx, ny, mx, my, npol, n_int = shape
+    for amp, sigma in STRONG:
+        v = synth.volts(n_int, 1, npol, nx, ny, seed=8, sigma=sigma, sources=[(0.137, 0.291, amp)])
+        w = synth.separable_weights(synth.half_sine(nx), synth.half_sine(ny)) if weights == "half_sine" \
+            else synth.random_weights(nx, ny, 5)
+        ref = oracle_beams(v, w, nx, ny, mx, my, npol, 1, n_int)
+        monkeypatch.setenv("FFTBF_FP32_PATH", "cov")
+        cov = rel_err_per_beam(run(v, w, nx, ny, mx, my, npol, 1, n_int), ref).max()
+        monkeypatch.setenv("FFTBF_FP32_PATH", "fft")
+        fft = rel_err_per_beam(run(v, w, nx, ny, mx, my, npol, 1, n_int), ref).max()
+        assert fft <= TOL_BEAM, (amp, sigma, fft)
+        assert cov <= 1e-6, (amp, sigma, cov, fft)
+
+
+@pytest.mark.parametrize("kind", ["half_sine", "random"])
+def test_weight_scale_and_range(kind, monkeypatch):
+    """Weights times a power of two give beams times its square, bit for bit, and what overflows is
+    infinite; a weight that is not finite takes the transform."""
+    monkeypatch.setenv("FFTBF_FP32_PATH", "cov")
+    shape = (4, 32, 4, 64, 2, 1, 64)
+    nx, ny, mx, my, npol, nfreq, n_int = shape
+    v, w = make_case(nx, ny, mx, my, npol, nfreq, n_int, n_int, weights=kind, seed=6)
+    one = run(v, w, *shape)
+    for e in (-40, 13, 40):
+        assert np.array_equal(run(v, w * np.float32(2.0 ** e), *shape), one * np.float32(2.0 ** (2 * e)))
+    assert np.all(np.isposinf(run(v, w * np.float32(2.0 ** 63), *shape)))
+    bad = w.copy()
+    bad[1, 3] = np.nan
+    got = run(v, bad, *shape)
+    monkeypatch.setenv("FFTBF_FP32_PATH", "fft")
+    assert np.array_equal(got, run(v, bad, *shape), equal_nan=True)
+
+
+def test_batch_mix_of_both_routes():
+    """220 snapshots per window: some arrays take the covariance and others the transform, real and
+    complex weights in both; each matches the oracle and is bit-identical alone."""
+    n_int, nwin = 110, 2
+    shapes = [(4, 256, 4, 512), (8, 64, 8, 128), (16, 16, 16, 32), (2, 512, 2, 1024), (1, 1024, 1, 2048),
+              (3, 128, 3, 256), (8, 64, 8, 128), (3, 128, 3, 256)]
+    arrays = []
+    for k, s in enumerate(shapes):
+        v, w = make_case(*s, 2, 1 + k % 3, n_int * nwin, n_int, weights="random" if k % 2 else "half_sine",
+                         seed=80 + k)
+        arrays.append((s, v, w))
+    plans = [fb.plan_create(*s, 2, v.shape[1], n_int, weights=w) for s, v, w in arrays]
+    with fb.batch_create(plans) as b:
+        steps = [fb.batch_tuned_steps(b, i) for i in range(len(plans))]
+    for p in plans:
+        p.close()
+    assert 64 in steps and any(t != 64 for t in steps), steps
+    mix = _batch(arrays, n_int, nwin, torch.cuda.Stream())
+    for (s, v, w), g in zip(arrays, mix):
+        ref = oracle_beams(v, w, *s, 2, v.shape[1], n_int)
+        assert rel_err_per_beam(g, ref).max() <= TOL_BEAM, s
+        assert np.array_equal(g, _batch([(s, v, w)], n_int, nwin)[0]), s
+
+
+@pytest.mark.parametrize("shape", [(4, 512, 4, 1024), (16, 64, 4, 128), (64, 32, 8, 64), (32, 16, 2, 32)],
+                         ids=lambda s: "x".join(map(str, s)))
+@pytest.mark.parametrize("weight", [0.7, 0.7 + 0.3j])
+def test_many_pairs_of_one_separation(shape, weight, monkeypatch):
+    """More than 1024 feed pairs of one separation, up to 16384 with co-added E-W rows: equal weights
+    that are no short binary fractions and a strong source make every product's part below a unit
+    of V alike, so that they add up. The bounds are those of the strong-source test; FP64 route."""
+    monkeypatch.setenv("FFTBF_FP32_PATH", "cov")
+    nx, ny, mx, my = shape
+    n_int = 64
+    v = synth.volts(n_int, 1, 1, nx, ny, seed=4, sigma=0.3, sources=[(0.0, 0.0, 7.0)])
+    w = np.full((nx, ny), weight, np.complex64)
+    got = run(v, w, nx, ny, mx, my, 1, 1, n_int)
+    ref = oracle_beams(v, w, nx, ny, mx, my, 1, 1, n_int)
+    assert rel_err_per_beam(got, ref).max() <= 1e-6
