@@ -1200,9 +1200,18 @@ static int corr_map(CorrJob* j) {
                                  (cuuint64_t)j->nant * a.npol * a.nfreq};
   const cuuint32_t box[4] = {128, (cuuint32_t)a.npol, 1, (cuuint32_t)(KS / a.npol)};
   const cuuint32_t one[4] = {1, 1, 1, 1};
-  const CUresult r = encode(&j->map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<uint8_t*>(a.volts), dims,
-                            strides, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  auto make = [&] {
+    return encode(&j->map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<uint8_t*>(a.volts), dims, strides,
+                  box, one, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  };
+  CUresult r = make();
+  if (r == CUDA_ERROR_INVALID_CONTEXT) {               // a thread's first call: the runtime binds its
+    int dev = 0;                                       // context only with work of its own
+    FFTBF_CUDA_TRY(cudaGetDevice(&dev));
+    FFTBF_CUDA_TRY(cudaSetDevice(dev));
+    r = make();
+  }
   if (r != CUDA_SUCCESS) return set_error(FFTBF_ECUDA, "cuTensorMapEncodeTiled failed (%d)", (int)r);
   return FFTBF_OK;
 }

@@ -310,3 +310,31 @@ def test_many_pairs_of_one_separation(shape, weight, monkeypatch):
     got = run(v, w, nx, ny, mx, my, 1, 1, n_int)
     ref = oracle_beams(v, w, nx, ny, mx, my, 1, 1, n_int)
     assert rel_err_per_beam(got, ref).max() <= 1e-6
+
+
+def test_first_call_of_a_thread():
+    """A host thread whose first CUDA call is the covariance route: the tensor map needs a context,
+    which the runtime has not bound to the thread yet."""
+    import threading
+    shape = (8, 64, 8, 128)
+    plan = fb.plan_create(*shape, 2, 1, 320)
+    v = torch.randint(0, 256, (320 * 2 * 512,), dtype=torch.uint8, device="cuda")
+    want, got = (torch.empty((1, 1, 8, 128), device="cuda") for _ in range(2))
+    errors = []
+    fb.execute(plan, v, 320, want)
+    stream = torch.cuda.current_stream()
+    torch.cuda.synchronize()
+
+    def work():
+        try:
+            fb.execute(plan, v, 320, got, stream=stream)
+        except Exception as e:  # noqa: BLE001 - reported below
+            errors.append(e)
+
+    t = threading.Thread(target=work)
+    t.start()
+    t.join()
+    assert not errors, errors[0]
+    fb.plan_sync(plan)
+    plan.close()
+    assert torch.equal(got, want)
