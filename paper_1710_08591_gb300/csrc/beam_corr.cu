@@ -77,6 +77,7 @@ constexpr int DS = 72;                   // pairs per staged diagonal (8 x 8, co
 constexpr float GRID = 12582912.f;       // 1.5 2^23: sums started here are whole numbers
 constexpr int MAXNS = 6, MAXNR = 3;
 constexpr int RAW = KS * 128;            // staged voltages of one operand: 64 snapshots x 128 feeds
+constexpr int SMEM_MAX = 227 * 1024 - 1024;   // dynamic; static: the barriers
 constexpr uint64_t WAIT_NS = 1000000000ull;
 // barriers: FULL/EMPTY per stage; accumulators done (RD, ID) and drained (RF, IF), V of
 // the other CTA ready (PV) and read by it (PE); raw voltages staged and read (RAWF, RAWE)
@@ -1171,11 +1172,10 @@ bool corr_sizes(const CorrJob* jobs, int n, CorrSizes* out) {
     s.tab = std::max(s.tab, tw_len(j.a.my) + tw_len(j.a.mx));
   }
   s.stg = (s.stg + 3) & ~3;
-  const int most = 227 * 1024 - 1024;                  // static shared memory: the barriers
   // the voltages' ring first (their latency is the longest), then operand stages
   s.nr = s.tma ? 2 : 0;
   s.ns = corr::MAXNS;
-  while (s.ns >= 2 && lay_of(s).total > most) --s.ns;
+  while (s.ns >= 2 && lay_of(s).total > corr::SMEM_MAX) --s.ns;
   *out = s;
   return s.ns >= 2;
 }
@@ -1229,7 +1229,9 @@ int corr_launch(CorrParams& p, int nsm, cudaStream_t st) {
   if (p.total <= 0) return FFTBF_OK;
   const int smem = std::max(lay_of(p.s).total, 120 * 1024);   // one CTA per SM: all tensor memory
   auto kern = p.s.cplx ? beams_corr_kernel<true> : beams_corr_kernel<false>;
-  FFTBF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  // The limit belongs to the kernel, not to this launch: every thread sets the same one, so that none
+  // takes it below what another is about to launch with.
+  FFTBF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, corr::SMEM_MAX));
   const int64_t pairs = std::min<int64_t>(p.total, nsm / 2);
   kern<<<(unsigned)(2 * pairs), corr::NT, smem, st>>>(p);
   FFTBF_CUDA_TRY(cudaGetLastError());

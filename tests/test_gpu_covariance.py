@@ -338,3 +338,36 @@ def test_first_call_of_a_thread():
     fb.plan_sync(plan)
     plan.close()
     assert torch.equal(got, want)
+
+
+def test_launches_of_different_sizes_from_several_threads(monkeypatch):
+    """Threads that launch lattices of different shared-memory sizes at once: the kernel's limit is
+    the same for all, so no launch is refused."""
+    import threading
+    monkeypatch.setenv("FFTBF_FP32_PATH", "cov")
+    shapes = [(4, 256, 4, 512), (1, 16, 1, 32), (8, 64, 8, 128), (2, 32, 2, 64)]
+    jobs, errors = [], []
+    for k, s in enumerate(shapes):
+        v, _ = make_case(*s, 1, 1, 32, 32, seed=k)
+        dv = torch.from_numpy(np.ascontiguousarray(v).reshape(-1)).cuda()
+        jobs.append((fb.plan_create(*s, 1, 1, 32), dv, torch.empty((1, 1, s[2], s[3]), device="cuda"),
+                     torch.cuda.Stream()))
+    torch.cuda.synchronize()
+
+    def work(plan, dv, out, st):
+        try:
+            for _ in range(1500):
+                fb.execute(plan, dv, 32, out, stream=st)
+        except Exception as e:  # noqa: BLE001 - reported below
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=j) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    for j in jobs:
+        fb.plan_sync(j[0])
+        j[0].close()
+    assert not errors, errors[0]
