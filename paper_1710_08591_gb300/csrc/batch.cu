@@ -501,8 +501,8 @@ fftbf_batch* fftbf_batch_create(fftbf_plan* const* plans, int n) {
     cudaSetDevice(prev);
     return nullptr;
   }
+  // the kernel's limit stays as set above: it holds for the launches of every batch and server
   bb->smem = std::max<size_t>(max_smem, 16);
-  cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bb->smem);
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel, kThreads, bb->smem);
   bb->grid_per_sm = std::max(1, per_sm);

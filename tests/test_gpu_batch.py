@@ -155,3 +155,25 @@ def test_batch_rejects_unsupported_shape():
         with pytest.raises(fb.FftbfError) as e:
             fb.batch_create([p])
         assert e.value.code == -5
+
+
+def test_an_earlier_batch_still_launches_after_a_smaller_one():
+    """The batch kernel's shared-memory limit holds for all batches: making one whose items need less,
+    or none of the kernel at all (arrays through the covariance), leaves an earlier one as it was."""
+    def plan(shape, n_int):
+        return fb.plan_create(*shape, 2, 4, n_int)
+
+    big = plan((4, 256, 4, 512), 32)
+    v = torch.randint(0, 256, (64 * 4 * 2 * 1024,), dtype=torch.uint8, device="cuda")
+    outs = [torch.full((2, 4, 4, 512), float("nan"), device="cuda") for _ in range(3)]
+    others = [plan((16, 16, 16, 32), 16), plan((8, 64, 8, 128), 320)]
+    with fb.batch_create([big]) as b:
+        fb.batch_execute(b, [v], 64, [outs[0]], None)
+        for o, p in zip(outs[1:], others):
+            with fb.batch_create([p]):
+                fb.batch_execute(b, [v], 64, [o], None)
+        torch.cuda.synchronize()
+    for p in [big] + others:
+        fb.plan_sync(p)
+        p.close()
+    assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
