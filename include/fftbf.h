@@ -227,7 +227,10 @@ int fftbf_execute_host(fftbf_plan* plan, const uint8_t* volts_host, int64_t T,
  * Supported shapes (pad_x x pad_y, pad_y >= ny):
  * 4x512, 8x128, 16x32, 2x1024, 1x2048, 3x256 (the N-S axis padded to twice the next
  * power of two of 256, 64, 16, 512, 1024, 128 feeds); others give FFTBF_EUNSUPPORTED.
- * The plans must outlive the batch, be on one device and not change precision.
+ * The plans must outlive the batch, be on one device and not change precision. fftbf_plan_sync of a
+ * plan waits for the last call of each batch that holds it, and returns FFTBF_ETIMEOUT if a device
+ * wait of a launch with that plan's array in it ran out (the other arrays of that launch are then
+ * incomplete too, and their plans report it as well).
  */
 typedef struct fftbf_batch fftbf_batch;
 /* n plans (1..64); allocates the work table and runs the autotuner. NULL on error. */

@@ -298,6 +298,7 @@ struct fftbf_batch {
   unsigned long long* d_counter = nullptr;
   size_t smem = 0;
   int grid_per_sm = 2;
+  cudaEvent_t done = nullptr;      // after the last launch; the plans wait for it in fftbf_plan_sync
   // graph of (counter reset + kernel) for the current job table
   cudaGraphExec_t exec = nullptr;
   cudaStream_t exec_stream = nullptr;
@@ -413,6 +414,7 @@ fftbf_batch* fftbf_batch_create(fftbf_plan* const* plans, int n) {
   cudaError_t e = cudaMalloc(&bb->d_jobs, sizeof(BatchJob) * bt::kMaxJobs);
   if (e == cudaSuccess) e = cudaMalloc(&bb->d_counter, sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaMalloc(&bb->d_cjobs, sizeof(CorrJob) * bt::kMaxJobs);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&bb->done, cudaEventDisableTiming);
   // shared memory: the largest item footprint over the plans and their S candidates
   bb->smem = 200 * 1024;
   if (e == cudaSuccess)
@@ -514,6 +516,7 @@ fftbf_batch* fftbf_batch_create(fftbf_plan* const* plans, int n) {
     return (double)p->n_int * p->npol * p->mx * p->my * std::log2((double)p->my + 1.0);
   };
   std::stable_sort(bb->order.begin(), bb->order.end(), [&](int x, int y) { return cost(x) > cost(y); });
+  for (auto* p : bb->plans) p->batch_events.push_back(bb->done);
   cudaSetDevice(prev);
   return bb;
 }
@@ -580,8 +583,10 @@ int fftbf_batch_execute(fftbf_batch* bb, const uint8_t* const* volts_dev, int64_
   if (st == nullptr) {
     // the legacy default stream cannot be captured: upload the table and launch directly
     if (bb->exec) { cudaGraphExecDestroy(bb->exec); bb->exec = nullptr; }
-    const int rc = upload();
-    return rc == FFTBF_OK ? launch_jobs(bb, total, st) : rc;
+    int rc = upload();
+    if (rc == FFTBF_OK) rc = launch_jobs(bb, total, st);
+    if (rc == FFTBF_OK) FFTBF_CUDA_TRY(cudaEventRecord(bb->done, st));
+    return rc;
   }
   const bool same = bb->exec && bb->exec_stream == st && bb->exec_T == T && bb->exec_ptrs == ptrs;
   if (!same) {
@@ -603,6 +608,7 @@ int fftbf_batch_execute(fftbf_batch* bb, const uint8_t* const* volts_dev, int64_
     bb->exec_ptrs = ptrs;
   }
   FFTBF_CUDA_TRY(cudaGraphLaunch(bb->exec, st));
+  FFTBF_CUDA_TRY(cudaEventRecord(bb->done, st));
   return FFTBF_OK;
 }
 
@@ -628,7 +634,15 @@ void fftbf_batch_destroy(fftbf_batch* bb) {
   int prev = 0;
   cudaGetDevice(&prev);
   cudaSetDevice(bb->device);
-  if (bb->exec_stream) cudaStreamSynchronize(bb->exec_stream);
+  if (bb->done) {
+    cudaEventSynchronize(bb->done);
+    for (auto* p : bb->plans) {
+      auto& v = p->batch_events;
+      const auto at = std::find(v.begin(), v.end(), bb->done);
+      if (at != v.end()) v.erase(at);
+    }
+    cudaEventDestroy(bb->done);
+  }
   if (bb->exec) cudaGraphExecDestroy(bb->exec);
   cudaFree(bb->d_jobs);
   cudaFree(bb->d_counter);

@@ -326,6 +326,7 @@ int fftbf_plan_sync(fftbf_plan* p) {
   if (!p) return set_error(FFTBF_EINVAL, "null plan");
   DeviceGuard g(p->device);
   for (cudaStream_t st : p->streams_used) FFTBF_CUDA_TRY(cudaStreamSynchronize(st));
+  for (cudaEvent_t e : p->batch_events) FFTBF_CUDA_TRY(cudaEventSynchronize(e));
   if (p->pipe.copy) FFTBF_CUDA_TRY(cudaStreamSynchronize(p->pipe.copy));
   for (int k = 0; k < HostPipe::kCopyStreams - 1; ++k)
     if (p->pipe.copy_extra[k]) FFTBF_CUDA_TRY(cudaStreamSynchronize(p->pipe.copy_extra[k]));

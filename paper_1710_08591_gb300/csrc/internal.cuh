@@ -226,4 +226,5 @@ struct fftbf_plan {
   float tc_scale = 1.f;
   int* d_err = nullptr;           // device error word of bounded waits
   std::vector<cudaStream_t> streams_used;
+  std::vector<cudaEvent_t> batch_events;   // of the batches that hold the plan: after their last launch
 };

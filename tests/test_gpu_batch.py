@@ -177,3 +177,26 @@ def test_an_earlier_batch_still_launches_after_a_smaller_one():
         fb.plan_sync(p)
         p.close()
     assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
+
+
+@pytest.mark.parametrize("n_int", [32, 320])
+def test_plan_sync_waits_for_a_batch(n_int):
+    """fftbf_plan_sync returns only after the batch's work on a non-blocking stream, for plans of both
+    routes, also when the batch's call replays its graph and after one of two batches is gone."""
+    shape, nwin = (8, 64, 8, 128), 2
+    plan = fb.plan_create(*shape, 2, 2, n_int)
+    v = torch.randint(0, 256, (nwin * n_int * 2 * 2 * 512,), dtype=torch.uint8, device="cuda")
+    out = torch.empty((nwin, 2, 8, 128), device="cuda")
+    st = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with fb.batch_create([plan]) as a:
+        with fb.batch_create([plan]) as b:
+            fb.batch_execute(b, [v], nwin * n_int, [out], st)
+        for _ in range(2):
+            with torch.cuda.stream(st):
+                torch.cuda._sleep(50_000_000)              # some 25 ms
+            fb.batch_execute(a, [v], nwin * n_int, [out], st)
+            assert not st.query()
+            fb.plan_sync(plan)
+            assert st.query()
+    plan.close()
