@@ -1132,7 +1132,9 @@ bool corr_make_job(const BeamArgs& a, CorrJob* J) {
   j.nt = (j.np + 255) / 256;
   const int64_t nsnap = (int64_t)a.n_int * a.npol;
   j.nch = (int)((nsnap + corr::KS - 1) / corr::KS);
-  j.tma = (a.ny & 15) == 0 && (reinterpret_cast<uintptr_t>(a.volts) & 15) == 0 && KS % a.npol == 0;
+  // TMA coordinates are 32 bits wide: a call of more samples loads them directly
+  j.tma = (a.ny & 15) == 0 && (reinterpret_cast<uintptr_t>(a.volts) & 15) == 0 && KS % a.npol == 0 &&
+          a.nwin * a.n_int <= INT32_MAX - KS;
   j.nitems = a.nwin * a.nfreq;
   // Units of V. With weights below 2 (w_exp) a product with its mirror is below 2 128 4 2^ns; a unit
   // is 2^-19 of that, and with n = nx ny ceil(nx / mx) feed pairs of one separation above 1024 2^e
@@ -1324,3 +1326,20 @@ int corr_plan_jobs(std::vector<CorrJob>& jobs, const CorrJob* d_table, int* err,
 }
 
 }  // namespace fftbf
+
+// How a call of nwin windows at address `volts` would bring its voltages (tests; host only): 1 by TMA,
+// 0 by direct loads, -1 if the kernel does not take the lattice.
+extern "C" int fftbf_corr_staging(int nx, int ny, int pad_x, int pad_y, int npol, int nfreq, int n_int,
+                                  int64_t nwin, uint64_t volts) {
+  fftbf::BeamArgs a{};
+  float4 here;
+  a.cw = &here;
+  a.nx = nx; a.ny = ny; a.mx = pad_x; a.my = pad_y;
+  a.npol = npol; a.nfreq = nfreq; a.n_int = n_int;
+  a.nyf = std::min(ny, pad_y);
+  a.real_w = 1;
+  a.nwin = nwin;
+  a.volts = reinterpret_cast<const uint8_t*>(volts);
+  fftbf::CorrJob j;
+  return fftbf::corr_make_job(a, &j) ? j.tma : -1;
+}

@@ -55,3 +55,20 @@ def test_nibbles_as_e4m3():
         nib = n & 15
         byte = abs((nib ^ 8) - 8) | ((nib << 4) & 0x80)
         assert e4m3(byte) == n * 2.0 ** -9
+
+
+@pytest.mark.parametrize("n_int,nwin,want", [
+    (64, 4, 1), (64, (2 ** 31 - 65) // 64, 1), (64, 2 ** 31 // 64, 0), (1 << 16, 1 << 16, 0), (384, 2 ** 40, 0)])
+def test_calls_past_32_bits_of_samples_load_directly(n_int, nwin, want):
+    """A TMA coordinate has 32 bits: calls whose sample index does not fit take the direct loads (the
+    same bits), not zeros past the wrap."""
+    import ctypes
+
+    import paper_1710_08591_gb300 as fb
+    fb.build()
+    f = fb.lib().fftbf_corr_staging
+    f.restype = ctypes.c_int
+    f.argtypes = [ctypes.c_int] * 7 + [ctypes.c_int64, ctypes.c_uint64]
+    assert f(1, 32, 1, 64, 1, 1, n_int, nwin, 1 << 20) == want
+    assert f(1, 32, 1, 64, 1, 1, n_int, nwin, (1 << 20) + 1) == 0          # off a 16-byte boundary
+    assert f(1, 33, 1, 64, 1, 1, n_int, nwin, 1 << 20) == 0                # rows of 33 feeds
