@@ -701,57 +701,57 @@ __device__ __forceinline__ void store_units(const uint4 (&x)[NE], unsigned char*
 // Columns that are the rows themselves (a full diagonal tile) are not staged again.
 __device__ __forceinline__ bool separate_cols(int I, int J, int cols) { return I != J || cols != 256; }
 
-// From voltages staged by TMA: the 128-byte swizzle moves 16-byte unit fb of row k to fb ^ (k & 7),
-// so eight lanes reading one unit of eight rows touch 128 distinct bytes.
-__device__ __forceinline__ void produce_staged(const CorrParams& P, unsigned char* raw,
-                                               unsigned char* ring, uint64_t* bars,
-                                               volatile int* abort_sm, int t, int64_t pair,
-                                               int64_t npairs) {
-  const int lane = t & 31, NS = P.s.ns, NR = P.s.nr, grp = t >> 7;
-  const int k = (t & 7) + 8 * ((t >> 6) & 1), fb = (t >> 3) & 7;
-  ring += (t & 7) * 16 + ((t >> 6) & 1) * LBO + fb * SBO;
-  raw += k * 128 + ((fb ^ (k & 7)) << 4);
-  const uint32_t full0 = map_rank(tc::smem_u32(bars + FULL), 0);
-  int slot = 0, rs = 0, turn = 0;                      // of the current stage
+// Where a producer stands: the operand stage (slot, par) and whose turn it is, the staged voltages
+// (rs, rpar).
+struct ProdState {
+  int slot = 0, turn = 0, rs = 0;
   uint32_t par = 1, rpar = 0;
-  int job = 0;
-  for (int64_t item = pair; item < P.total; item += npairs) {
-    const CorrJob& J = find_job(P, item, job);
-    const int nt = J.nt, np = J.np, nsnap = J.a.n_int * J.a.npol;
-    for (int I = 0; I < nt; ++I)
-      for (int Jc = I; Jc < nt; ++Jc) {
-        const int cols = tile_cols(np, Jc);
-        const bool hasb = separate_cols(I, Jc, cols) && 16 * fb < cols / 2;
-        for (int left = nsnap; left > 0; left -= KS) {
-          if (turn == grp) {
-            const bool ok = wait_pair(bars + RAWF + rs, rpar, abort_sm) && wait_pair(bars + EMPTY + slot, par, abort_sm);
-            if (!ok) corr_fail(P, abort_sm);
-            if (!__all_sync(0xffffffffu, ok)) return;
-            const unsigned char* src = raw + rs * (2 * RAW);
-            unsigned char* dst = ring + slot * STAGE;
-            uint4 x[NE], y[NE];
+};
+
+// An item's stages from voltages staged by TMA: the 128-byte swizzle moves 16-byte unit fb of row k to
+// fb ^ (k & 7), so eight lanes reading one unit of eight rows touch 128 distinct bytes.
+__device__ __forceinline__ bool produce_staged(const CorrParams& P, const CorrJob& J,
+                                               const unsigned char* raw, unsigned char* ring,
+                                               uint64_t* bars, volatile int* abort_sm, int t,
+                                               uint32_t full0, ProdState& S) {
+  const int lane = t & 31, grp = t >> 7, k = (t & 7) + 8 * ((t >> 6) & 1), fb = (t >> 3) & 7;
+  raw += k * 128 + ((fb ^ (k & 7)) << 4);
+  const int nt = J.nt, np = J.np, nsnap = J.a.n_int * J.a.npol;
+  for (int I = 0; I < nt; ++I)
+    for (int Jc = I; Jc < nt; ++Jc) {
+      const int cols = tile_cols(np, Jc);
+      const bool hasb = separate_cols(I, Jc, cols) && 16 * fb < cols / 2;
+      for (int left = nsnap; left > 0; left -= KS) {
+        if (S.turn == grp) {
+          const bool ok = wait_pair(bars + RAWF + S.rs, S.rpar, abort_sm) &&
+                          wait_pair(bars + EMPTY + S.slot, S.par, abort_sm);
+          if (!ok) corr_fail(P, abort_sm);
+          if (!__all_sync(0xffffffffu, ok)) return false;
+          const unsigned char* src = raw + S.rs * (2 * RAW);
+          unsigned char* dst = ring + S.slot * STAGE;
+          uint4 x[NE], y[NE];
 #pragma unroll
-            for (int e = 0; e < NE; ++e) {
-              x[e] = *reinterpret_cast<const uint4*>(src + e * (RAW / NE));
-              if (hasb) y[e] = *reinterpret_cast<const uint4*>(src + RAW + e * (RAW / NE));
-              if (k + 16 * e >= left) x[e] = y[e] = make_uint4(0u, 0u, 0u, 0u);   // the next window's
-            }
-            __syncwarp();
-            if (lane == 0) tc::mbar_arrive(bars + RAWE + rs);
-            store_units(x, dst);
-            if (hasb) store_units(y, dst + 2 * TILE);
-            tc::fence_proxy_async_smem();
-            __syncwarp();
-            if (lane == 0) arrive_cluster(full0 + 8 * slot);
+          for (int e = 0; e < NE; ++e) {
+            x[e] = *reinterpret_cast<const uint4*>(src + e * (RAW / NE));
+            if (hasb) y[e] = *reinterpret_cast<const uint4*>(src + RAW + e * (RAW / NE));
+            if (k + 16 * e >= left) x[e] = y[e] = make_uint4(0u, 0u, 0u, 0u);   // the next window's
           }
-          turn ^= 1;
-          if (++slot == NS) { slot = 0; par ^= 1; }
-          if (++rs == NR) { rs = 0; rpar ^= 1; }
+          __syncwarp();
+          if (lane == 0) tc::mbar_arrive(bars + RAWE + S.rs);
+          store_units(x, dst);
+          if (hasb) store_units(y, dst + 2 * TILE);
+          tc::fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) arrive_cluster(full0 + 8 * S.slot);
         }
+        S.turn ^= 1;
+        if (++S.slot == P.s.ns) { S.slot = 0; S.par ^= 1; }
+        if (++S.rs == P.s.nr) { S.rs = 0; S.rpar ^= 1; }
       }
-  }
+    }
+  return true;
 }
-// One thread: the TMA tiles of every stage, rows and (if separate) columns.
+// One thread: the TMA tiles of every stage of the jobs that take them, rows and (if separate) columns.
 __device__ __forceinline__ void stage_volts(const CorrParams& P, unsigned char* raw, uint64_t* bars,
                                             volatile int* abort_sm, uint32_t rank, int64_t pair,
                                             int64_t npairs) {
@@ -765,6 +765,7 @@ __device__ __forceinline__ void stage_volts(const CorrParams& P, unsigned char* 
   const CorrJob* last = nullptr;
   for (int64_t item = pair; item < P.total && ok; item += npairs) {
     const CorrJob& J = find_job(P, item, job);
+    if (!J.tma) continue;
     if (P.table && &J != last) acquire_map(&J.map);
     last = &J;
     const int nt = J.nt, np = J.np, npol = J.a.npol, nch = J.nch;
@@ -794,58 +795,69 @@ __device__ __forceinline__ void stage_volts(const CorrParams& P, unsigned char* 
 }
 
 // From global memory, byte by byte where the lattice or the pointer is not a multiple of 16 bytes.
-__device__ __forceinline__ void produce_direct(const CorrParams& P, unsigned char* ring, uint64_t* bars,
+__device__ __forceinline__ bool produce_direct(const CorrParams& P, const CorrJob& J, int64_t item,
+                                               unsigned char* ring, uint64_t* bars,
                                                volatile int* abort_sm, int t, uint32_t rank,
-                                               int64_t pair, int64_t npairs) {
-  const int lane = t & 31, NS = P.s.ns, grp = t >> 7;
-  const int k = (t & 7) + 8 * ((t >> 6) & 1), fb = (t >> 3) & 7;
-  ring += (t & 7) * 16 + ((t >> 6) & 1) * LBO + fb * SBO;
-  const uint32_t full0 = map_rank(tc::smem_u32(bars + FULL), 0);
-  int slot = 0, turn = 0, job = 0;
-  uint32_t par = 1;
-  for (int64_t item = pair; item < P.total; item += npairs) {
-    const CorrJob& J = find_job(P, item, job);
-    const BeamArgs& a = J.a;
-    const int nt = J.nt, np = J.np, nsnap = a.n_int * a.npol, nyp = J.nyp, ny = J.ny, nx = a.nx;
-    const uint8_t* begin = a.volts;
-    const uint8_t* end = begin + a.nwin * a.n_int * a.nfreq * a.npol * (int64_t)J.nant;
-    const uint8_t* ivol = item_volts(a, item - J.item0, J.nant);
-    for (int I = 0; I < nt; ++I)
-      for (int Jc = I; Jc < nt; ++Jc) {
-        const int cols = tile_cols(np, Jc);
-        const bool hasb = separate_cols(I, Jc, cols) && 16 * fb < cols / 2;
-        int off[2] = {0, 0}, cnt[2] = {0, 0};          // feed offset and live feeds of the units
-        auto unit = [&](int s, int b) {
-          const int ix = s / nyp, iy = s - ix * nyp;
-          off[b] = ix * ny + iy;
-          cnt[b] = ix < nx ? max(0, min(16, ny - iy)) : 0;
-        };
-        unit(256 * I + 128 * (int)rank + 16 * fb, 0);
-        if (hasb) unit(256 * Jc + (int)rank * (cols / 2) + 16 * fb, 1);
-        for (int g = k; g - k < nsnap; g += KS) {
-          if (turn == grp) {
-            const bool ok = wait_pair(bars + EMPTY + slot, par, abort_sm);
-            if (!ok) corr_fail(P, abort_sm);
-            if (!__all_sync(0xffffffffu, ok)) return;
+                                               uint32_t full0, ProdState& S) {
+  const int lane = t & 31, grp = t >> 7, k = (t & 7) + 8 * ((t >> 6) & 1), fb = (t >> 3) & 7;
+  const BeamArgs& a = J.a;
+  const int nt = J.nt, np = J.np, nsnap = a.n_int * a.npol, nyp = J.nyp, ny = J.ny, nx = a.nx;
+  const uint8_t* begin = a.volts;
+  const uint8_t* end = begin + a.nwin * a.n_int * a.nfreq * a.npol * (int64_t)J.nant;
+  const uint8_t* ivol = item_volts(a, item - J.item0, J.nant);
+  for (int I = 0; I < nt; ++I)
+    for (int Jc = I; Jc < nt; ++Jc) {
+      const int cols = tile_cols(np, Jc);
+      const bool hasb = separate_cols(I, Jc, cols) && 16 * fb < cols / 2;
+      int off[2] = {0, 0}, cnt[2] = {0, 0};            // feed offset and live feeds of the units
+      auto unit = [&](int s, int b) {
+        const int ix = s / nyp, iy = s - ix * nyp;
+        off[b] = ix * ny + iy;
+        cnt[b] = ix < nx ? max(0, min(16, ny - iy)) : 0;
+      };
+      unit(256 * I + 128 * (int)rank + 16 * fb, 0);
+      if (hasb) unit(256 * Jc + (int)rank * (cols / 2) + 16 * fb, 1);
+      for (int g = k; g - k < nsnap; g += KS) {
+        if (S.turn == grp) {
+          const bool ok = wait_pair(bars + EMPTY + S.slot, S.par, abort_sm);
+          if (!ok) corr_fail(P, abort_sm);
+          if (!__all_sync(0xffffffffu, ok)) return false;
 #pragma unroll 1
-            for (int b = 0; b < (hasb ? 2 : 1); ++b) {
-              uint4 x[NE];
+          for (int b = 0; b < (hasb ? 2 : 1); ++b) {
+            uint4 x[NE];
 #pragma unroll
-              for (int e = 0; e < NE; ++e) {
-                const int ge = g + 16 * e;
-                x[e] = load16_any(ivol + snap_offset(a, ge, J.nant) + (b ? off[1] : off[0]),
-                                  ge < nsnap ? (b ? cnt[1] : cnt[0]) : 0, begin, end);
-              }
-              store_units(x, ring + slot * STAGE + b * (2 * TILE));
+            for (int e = 0; e < NE; ++e) {
+              const int ge = g + 16 * e;
+              x[e] = load16_any(ivol + snap_offset(a, ge, J.nant) + (b ? off[1] : off[0]),
+                                ge < nsnap ? (b ? cnt[1] : cnt[0]) : 0, begin, end);
             }
-            tc::fence_proxy_async_smem();
-            __syncwarp();
-            if (lane == 0) arrive_cluster(full0 + 8 * slot);
+            store_units(x, ring + S.slot * STAGE + b * (2 * TILE));
           }
-          turn ^= 1;
-          if (++slot == NS) { slot = 0; par ^= 1; }
+          tc::fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) arrive_cluster(full0 + 8 * S.slot);
         }
+        S.turn ^= 1;
+        if (++S.slot == P.s.ns) { S.slot = 0; S.par ^= 1; }
       }
+    }
+  return true;
+}
+
+// Each item by the way its own job allows: an array whose voltages cannot come by TMA does not slow
+// the others of its launch.
+__device__ __forceinline__ void produce(const CorrParams& P, const unsigned char* raw, unsigned char* ring,
+                                        uint64_t* bars, volatile int* abort_sm, int t, uint32_t rank,
+                                        int64_t pair, int64_t npairs) {
+  ring += (t & 7) * 16 + ((t >> 6) & 1) * LBO + ((t >> 3) & 7) * SBO;
+  const uint32_t full0 = map_rank(tc::smem_u32(bars + FULL), 0);
+  ProdState S;
+  int job = 0;
+  bool ok = true;
+  for (int64_t item = pair; item < P.total && ok; item += npairs) {
+    const CorrJob& J = find_job(P, item, job);
+    ok = J.tma ? produce_staged(P, J, raw, ring, bars, abort_sm, t, full0, S)
+               : produce_direct(P, J, item, ring, bars, abort_sm, t, rank, full0, S);
   }
 }
 
@@ -1039,10 +1051,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(corr::NT, 1)
     }
   } else if (warp < 8 + PROD / 32) {
     // ================================================= producers
-    if (P.s.tma)
-      produce_staged(P, smem + Y.raw, smem + Y.ring, bars, abort_sm, tid - EPI, pair, npairs);
-    else
-      produce_direct(P, smem + Y.ring, bars, abort_sm, tid - EPI, rank, pair, npairs);
+    produce(P, smem + Y.raw, smem + Y.ring, bars, abort_sm, tid - EPI, rank, pair, npairs);
   } else if (warp == 17 && lane == 0 && P.s.tma) {
     stage_volts(P, smem + Y.raw, bars, abort_sm, rank, pair, npairs);
   } else if ((warp == 16 || warp == 18) && rank == 0 && lane == 0) {
@@ -1159,10 +1168,9 @@ bool corr_make_job(const BeamArgs& a, CorrJob* J) {
 // Shared-memory sizes that hold every job of a launch; false if they do not fit.
 bool corr_sizes(const CorrJob* jobs, int n, CorrSizes* out) {
   CorrSizes s{};
-  s.tma = 1;
   for (int i = 0; i < n; ++i) {
     s.cplx |= !jobs[i].a.real_w;
-    s.tma &= jobs[i].tma;
+    s.tma |= jobs[i].tma;
   }
   for (int i = 0; i < n; ++i) {
     const CorrJob& j = jobs[i];
@@ -1218,9 +1226,10 @@ static int corr_map(CorrJob* j) {
   return FFTBF_OK;
 }
 
-// Prepare the jobs' tensor maps (when every job takes them).
-int corr_maps(CorrJob* jobs, int n, const CorrSizes& s) {
-  for (int i = 0; i < n && s.tma; ++i) {
+// Prepare the tensor maps of the jobs that take them.
+int corr_maps(CorrJob* jobs, int n) {
+  for (int i = 0; i < n; ++i) {
+    if (!jobs[i].tma) continue;
     const int rc = corr_map(jobs + i);
     if (rc != FFTBF_OK) return rc;
   }
@@ -1285,7 +1294,7 @@ int launch_beams_corr(const BeamArgs& a, int nsm, cudaStream_t st) {
   CorrParams p{};
   if (!corr_make_job(a, &p.one) || !corr_sizes(&p.one, 1, &p.s))
     return set_error(FFTBF_EUNSUPPORTED, "lattice too large for the covariance kernel");
-  const int rc = corr_maps(&p.one, 1, p.s);
+  const int rc = corr_maps(&p.one, 1);
   if (rc != FFTBF_OK) return rc;
   p.total = p.one.nitems;
   p.njobs = 1;
@@ -1297,9 +1306,9 @@ int launch_beams_corr(const BeamArgs& a, int nsm, cudaStream_t st) {
 int corr_plan_jobs(std::vector<CorrJob>& jobs, const CorrJob* d_table, int* err,
                    std::vector<CorrParams>* out) {
   out->clear();
-  std::stable_sort(jobs.begin(), jobs.end(), [](const CorrJob& x, const CorrJob& y) {
-    return (double)x.np * x.np * x.nch > (double)y.np * y.np * y.nch;
-  });
+  auto cost = [](const CorrJob& j) { return (j.tma ? 1.0 : 3.0) * j.np * j.np * j.nch; };
+  std::stable_sort(jobs.begin(), jobs.end(),
+                   [&](const CorrJob& x, const CorrJob& y) { return cost(x) > cost(y); });
   for (size_t i = 0; i < jobs.size();) {
     CorrParams p{};
     size_t n = 1;
@@ -1310,7 +1319,7 @@ int corr_plan_jobs(std::vector<CorrJob>& jobs, const CorrJob* d_table, int* err,
       p.s = s;
       ++n;
     }
-    const int rc = corr_maps(&jobs[i], (int)n, p.s);
+    const int rc = corr_maps(&jobs[i], (int)n);
     if (rc != FFTBF_OK) return rc;
     for (size_t k = i; k < i + n; ++k) {
       jobs[k].item0 = p.total;

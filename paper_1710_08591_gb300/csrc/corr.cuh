@@ -26,7 +26,7 @@ struct CorrSizes {      // shared-memory sizes, the largest over the launch's jo
   int ns, nr;           // operand stages, staged voltage tiles
   int wslots, vlen, stg, tab;
   int cplx;             // some weights are complex
-  int tma;              // every job's voltages are staged by TMA
+  int tma;              // some jobs' voltages are staged by TMA
 };
 struct CorrParams {
   CorrJob one;          // the only job, or
@@ -40,7 +40,7 @@ struct CorrParams {
 // Fill a job; false where the kernel does not take the lattice.
 bool corr_make_job(const BeamArgs& a, CorrJob* J);
 bool corr_sizes(const CorrJob* jobs, int n, CorrSizes* out);
-int corr_maps(CorrJob* jobs, int n, const CorrSizes& s);
+int corr_maps(CorrJob* jobs, int n);
 int corr_launch(CorrParams& p, int nsm, cudaStream_t st);
 constexpr int kCorrSteps = 64;   // snapshots per operand stage
 // Whether it beats the transform of every snapshot (split: the split-FP16 kernel).

@@ -371,3 +371,34 @@ def test_launches_of_different_sizes_from_several_threads(monkeypatch):
         fb.plan_sync(j[0])
         j[0].close()
     assert not errors, errors[0]
+
+
+def test_batch_of_staged_and_direct_voltages(monkeypatch):
+    """Aligned arrays beside one of 60-feed rows and one off a 16-byte boundary, several items of each
+    per CTA pair: every array's beams are the bits of its own call, and match the oracle."""
+    monkeypatch.setenv("FFTBF_FP32_PATH", "cov")
+    n_int, nwin = 160, 3
+    shapes = [(4, 256, 4, 512, 40), (8, 60, 8, 128, 33), (8, 64, 8, 128, 50), (4, 256, 4, 512, 3), (3, 100, 3, 256, 20)]
+    rng = np.random.default_rng(12)
+    plans, dvs, outs, vs = [], [], [], []
+    for k, (nx, ny, mx, my, nf) in enumerate(shapes):
+        w = synth.random_weights(nx, ny, k) if k in (2, 4) else None
+        plans.append(fb.plan_create(nx, ny, mx, my, 2, nf, n_int, weights=w))
+        v = rng.integers(0, 256, (nwin * n_int, nf, 2, nx, ny), dtype=np.uint8)
+        base = torch.empty(v.size + 16, dtype=torch.uint8, device="cuda")
+        dvs.append(base[5 * (k == 3):][:v.size])
+        dvs[-1].copy_(torch.from_numpy(v.reshape(-1)))
+        outs.append(torch.full((nwin, nf, mx, my), float("nan"), device="cuda"))
+        vs.append((v, w))
+    with fb.batch_create(plans) as b:
+        assert {fb.batch_tuned_steps(b, i) for i in range(len(plans))} == {64}
+        fb.batch_execute(b, dvs, nwin * n_int, outs, torch.cuda.Stream())
+        torch.cuda.synchronize()
+    for p, d, o, (v, w), s in zip(plans, dvs, outs, vs, shapes):
+        own = torch.empty_like(o)
+        fb.execute(p, d, nwin * n_int, own)
+        fb.plan_sync(p)
+        p.close()
+        assert torch.equal(o, own), s
+        ref = oracle_beams(np.ascontiguousarray(v[:n_int, :1]), w, *s[:4], 2, 1, n_int)
+        assert rel_err_per_beam(o[:1, :1].cpu().numpy(), ref).max() <= TOL_BEAM, s
