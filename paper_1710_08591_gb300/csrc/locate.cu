@@ -167,9 +167,12 @@ __device__ __forceinline__ float warp_sum_c(CSum v) {
 // advance a position by dy (in units of y) and renormalise fr into [0, 1), ih into [0, M)
 __device__ __forceinline__ void move(const LocAxis& ax, int* ih, float* fr, float dyM) {
   float f = *fr + dyM;
-  const float k = floorf(f);
+  float k = floorf(f);
   f -= k;
-  if (f >= 1.f) f = 0.f;                               // rounding of f - k at the top end
+  if (f >= 1.f) {                                      // a tiny step down from a beam: f - k rounds to 1
+    f = 0.f;
+    k += 1.f;
+  }
   *ih = mod_m(ax, *ih + (int)k);
   *fr = f;
 }

@@ -103,3 +103,28 @@ def test_localise_final_sum_over_sizes(nx, ny, mx, my):
     ref = oracle.localise(P, nx, ny, n_iter=5, n_taps=10)
     assert (np.abs((got[..., :2] - ref[..., :2] + 0.5) % 1.0 - 0.5) < 2e-6).all()
     assert np.allclose(got[..., 2], ref[..., 2], rtol=1e-5)
+
+
+@pytest.mark.parametrize("nx,ny,mx,my", [(3, 30, 5, 66), (2, 20, 3, 41), (3, 16, 5, 32), (5, 12, 9, 24)])
+def test_localise_step_of_rounding_size_on_a_beam(nx, ny, mx, my):
+    """A source exactly on an E-W beam: the Newton steps are of rounding size and of either sign, and
+    one just below the beam stays on it (it went one whole beam down). The other axis anywhere. The
+    oracle's estimate within the bounds of the other comparisons here."""
+    rng = np.random.default_rng(3)
+    nwin, nfreq = 6, 4
+    y0 = rng.random((nwin, nfreq))
+    B = np.arange(my) / my
+    row = np.abs(np.sum(np.exp(2j * np.pi * np.arange(ny) * (B[None, None, :, None] - y0[..., None, None])),
+                        axis=-1)) ** 2 / ny ** 2 + 0.05
+    P = np.repeat(row[:, :, None, :], mx, axis=2).astype(np.float32)
+    P[:, :, 0] *= 1.5                                                   # symmetric about E-W beam 0
+    P = np.roll(P, 2, axis=2)                                           # on beam 2
+    dP = torch.from_numpy(P).cuda()
+    out = torch.full((nwin, nfreq, 3), float("nan"), device="cuda")
+    with fb.plan_create(nx, ny, mx, my, 1, nfreq, 8) as plan:
+        fb.localise(plan, dP, nwin, out, n_iter=5, n_taps=10)
+        fb.plan_sync(plan)
+    got = out.cpu().numpy()
+    ref = oracle.localise(P, nx, ny, n_iter=5, n_taps=10)
+    assert (np.abs((got[..., :2] - ref[..., :2] + 0.5) % 1.0 - 0.5) < 2e-6).all()
+    assert np.allclose(got[..., 2], ref[..., 2], rtol=1e-5)
