@@ -14,10 +14,9 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <system_error>
-#include <thread>
 
 #include "internal.cuh"
+#include "same_bytes.cuh"
 
 namespace fftbf {
 
@@ -499,38 +498,6 @@ static int tt_sms(cudaStream_t) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
   return n > 0 ? n : 1;
-}
-
-// Whether two arrays of n bytes are the same. One core compares at about 25 GB/s: 360 us per call
-// for the u and v of 256 channels x 2048 pointings (4.2 MB each), more than the beams of 64 windows
-// take on the device (304 us). Arrays of 2 MB and more are shared among up to four threads, 1 MB
-// or more each (260 us for these two; a thread costs some 20 us to start). A piece whose thread
-// cannot start is compared here.
-static bool same_bytes(const void* a, const void* b, size_t n) {
-  constexpr size_t kPiece = 1u << 20;
-  constexpr int kMax = 4;
-  const char* x = static_cast<const char*>(a);
-  const char* y = static_cast<const char*>(b);
-  const int parts = (int)std::min<size_t>(kMax, std::max<size_t>(1, n / kPiece));
-  const size_t step = n / parts;
-  bool same[kMax] = {true, true, true, true};
-  std::thread th[kMax];
-  for (int i = 1; i < parts; ++i) {
-    const size_t o = i * step, len = i == parts - 1 ? n - o : step;
-    bool* r = &same[i];
-    try {
-      th[i] = std::thread([=] { *r = std::memcmp(x + o, y + o, len) == 0; });
-    } catch (const std::system_error&) {
-      *r = std::memcmp(x + o, y + o, len) == 0;
-    }
-  }
-  same[0] = std::memcmp(x, y, parts > 1 ? step : n) == 0;
-  bool all = same[0];
-  for (int i = 1; i < parts; ++i) {
-    if (th[i].joinable()) th[i].join();
-    all = all && same[i];
-  }
-  return all;
 }
 
 int tied_prepare(TiedTables& tt, int nx, int ny, int mx, int my, int nfreq, int n_tied,
