@@ -80,9 +80,10 @@ constexpr int RAW = KS * 128;            // staged voltages of one operand: 64 s
 constexpr int SMEM_MAX = 227 * 1024 - 1024;   // dynamic; static: the barriers
 constexpr uint64_t WAIT_NS = 1000000000ull;
 // barriers: FULL/EMPTY per stage; accumulators done (RD, ID) and drained (RF, IF), V of
-// the other CTA ready (PV) and read by it (PE); raw voltages staged and read (RAWF, RAWE)
+// the other CTA ready (PV) and read by it (PE); raw voltages staged and read (RAWF, RAWE); the
+// MMAs of an issuer that gave up (LR, LI)
 enum { RD = 0, ID, RF, IF, PV, PE, FULL, EMPTY = FULL + MAXNS, RAWF = EMPTY + MAXNS,
-       RAWE = RAWF + MAXNR, NBAR = RAWE + MAXNR };
+       RAWE = RAWF + MAXNR, LR = RAWE + MAXNR, LI, NBAR };
 }  // namespace corr
 
 namespace {
@@ -887,7 +888,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(corr::NT, 1)
   }
   if (tid == 0) {
     for (int i = 0; i < NBAR; ++i) {
-      uint32_t c = 1;                                  // MMA commits, PE
+      uint32_t c = 1;                                  // MMA commits, PV, PE
       if (i == RF || i == IF) c = 2 * EPI / 32;         // warps of both CTAs
       if (i >= FULL && i < FULL + MAXNS) c = 2 * PROD / 64;      // half of the producers
       if (i >= EMPTY && i < EMPTY + MAXNS) c = 2;      // commits of both issuers
@@ -1062,9 +1063,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(corr::NT, 1)
     const int done = im ? ID : RD, drained = im ? IF : RF;
     int slot = 0;
     uint32_t par = 0, tph = 1;                         // tph: parity of the drained barrier
-    int64_t tiles = 0;
     int job = 0;
-    bool ok = true;
+    bool ok = true, issued = false;
     for (int64_t item = pair; item < P.total && ok; item += npairs) {
       const CorrJob& J = find_job(P, item, job);
       const int nt = J.nt, np = J.np, nsnap = J.a.n_int * J.a.npol;
@@ -1082,6 +1082,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(corr::NT, 1)
           ok = wait_one(drained, tph);
           if (!ok) break;
           tc::fence_after_sync();
+          issued = true;
           for (int left = nsnap; left > 0; left -= KS) {
             ok = wait_one(FULL + slot, par);
             if (!ok) break;
@@ -1100,13 +1101,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(corr::NT, 1)
           if (!ok) break;
           commit_pair(bars + done);
           tph ^= 1;
-          ++tiles;
         }
     }
-    // every MMA issued must have completed before the pair frees its memory
-    if (tiles > 0) {
+    // every MMA issued, those of a tile given up half-way included, must have completed before the
+    // pair frees its memory
+    if (issued) {
       volatile int never = 0;
-      wait_pair(bars + done, (uint32_t)((tiles - 1) & 1), &never);
+      commit_pair(bars + (im ? LI : LR));
+      wait_pair(bars + (im ? LI : LR), 0, &never);
     }
   }
   __syncwarp();
