@@ -291,10 +291,16 @@ __global__ void __launch_bounds__(ttc::NT, 2) tied_tc_kernel(
         tc::bulk_g2s(stg + 2 * ttc::TILE + PT, pl + pt, PT, &full[st]);
       }
     }
-    if (!ok) atomicExch(&s_ok, 0);
+    if (!ok) {
+      atomicExch(&s_ok, 0);
+      // copies in flight must have landed before the CTA gives back its memory
+      for (int c = t > NS ? t - NS : 0; c < t; ++c)
+        tc::mbar_wait(&full[c % NS], (uint32_t)((c / NS) & 1), ttc::WAIT_NS);
+    }
   } else if (tid == 0) {
     bool ok = true;
-    for (int t = 0; t < total && ok; ++t) {
+    int t = 0;
+    for (; t < total; ++t) {
       const int st = t % NS;
       ok = tc::mbar_wait(&full[st], (uint32_t)((t / NS) & 1), ttc::WAIT_NS);
       if (!ok) break;
@@ -315,9 +321,9 @@ __global__ void __launch_bounds__(ttc::NT, 2) tied_tc_kernel(
       }
       tc::mma_commit(&empty[st]);
     }
-    if (ok && total > 0) {                          // the last commit covers every MMA
-      const int tl = total - 1;
-      ok = tc::mbar_wait(&empty[tl % NS], (uint32_t)((tl / NS) & 1), ttc::WAIT_NS);
+    if (t > 0) {                                    // the last commit covers every MMA issued
+      const int tl = t - 1;
+      ok = tc::mbar_wait(&empty[tl % NS], (uint32_t)((tl / NS) & 1), ttc::WAIT_NS) && ok;
     }
     if (!ok) atomicExch(&s_ok, 0);
   }
