@@ -402,3 +402,22 @@ def test_batch_of_staged_and_direct_voltages(monkeypatch):
         assert torch.equal(o, own), s
         ref = oracle_beams(np.ascontiguousarray(v[:n_int, :1]), w, *s[:4], 2, 1, n_int)
         assert rel_err_per_beam(o[:1, :1].cpu().numpy(), ref).max() <= TOL_BEAM, s
+
+
+@pytest.mark.parametrize("npol,n_int", [(1, 65536), (1, 65535), (2, 32768), (64, 1024)])
+def test_sums_of_65536_snapshots_are_exact(npol, n_int, monkeypatch):
+    """The tensor cores' sums of up to 65536 snapshots, near 2^23 and odd, to the last bit: one feed,
+    and two feeds whose beams are |x_0 +- x_1|^2, each as the rounding of the whole number to FP32."""
+    monkeypatch.setenv("FFTBF_FP32_PATH", "cov")
+    rng = np.random.default_rng(npol + n_int)
+    for spread in (0, 1, 4):                                           # all -8, mixed with -7, all signs
+        x = np.where(rng.random((n_int, npol, 2, 2)) < 0.9, -8, rng.integers(-8, -7 + spread * 2, (n_int, npol, 2, 2)))
+        x[n_int // 2, 0, 0, 0] = -7                                    # one odd term
+        for nf in (1, 2):
+            y = x[:, :, :nf]
+            v = ((y[..., 0] & 15) << 4 | (y[..., 1] & 15)).astype(np.uint8).reshape(n_int, 1, npol, 1, nf)
+            got = run(v, None, 1, nf, 1, nf, npol, 1, n_int)[0, 0, 0]
+            z = y.astype(np.int64)
+            for B in range(nf):
+                s = z.sum(axis=2) if B == 0 else z[:, :, 0] - z[:, :, 1]
+                assert got[B] == np.float32(int((s ** 2).sum())), (spread, nf, B)

@@ -178,3 +178,26 @@ def test_tensor_core_form_full_size(run, form, pipe, monkeypatch):
         assert rms <= rms_tol, (form, j, f, rms)
     assert rel_all.max() <= tol + TOL_BEAM, (form, float(rel_all.max()))
     assert prel.max() <= PARSEVAL[form], (form, float(prel.max()))
+
+
+@pytest.mark.parametrize("form", ["fp32", "fp16x3"])
+@pytest.mark.parametrize("route", ["cov", "fft"])
+def test_each_route_full_size(run, form, route, monkeypatch):
+    """The FP32-accurate forms by both their routes over the 8192-item launch, whatever the rule takes
+    at this window: the 4x256 transform and the split-FP16 kernel with several items per CTA, and the
+    covariance. Sampled slices against the oracle, every item against Parseval and the default route."""
+    monkeypatch.setenv("FFTBF_FP32_PATH", route)
+    beams = torch.full((NWIN, NFREQ, MX, MY), float("nan"), device="cuda")
+    with fb.plan_create(NX, NY, MX, MY, NPOL, NFREQ, NINT, weights=run["w"]) as plan:
+        if form == "fp16x3":
+            fb.plan_set_precision(plan, fb.PREC_TC_FP16X3)
+        fb.execute(plan, run["dvol"], T_DEV, beams)
+        fb.plan_sync(plan)
+    got = beams.cpu().numpy()
+    del beams
+    assert np.all(np.isfinite(got))
+    for j, f in SLICES:
+        ref = _oracle_slice(run, j, f)[0, 0]
+        assert (np.abs(got[j, f] - ref) / ref).max() <= TOL_BEAM, (j, f)
+    assert (np.abs(got - run["beams"]) / run["beams"]).max() <= 2 * TOL_BEAM
+    _check_parseval(run, got, form)
