@@ -1251,20 +1251,24 @@ int corr_launch(CorrParams& p, int nsm, cudaStream_t st) {
   return FFTBF_OK;
 }
 
-// Where the covariance beats the transform of every snapshot. Both are taken as microseconds of 608
-// work items (eight per CTA pair), measured on a GB300 from 16 to 768 snapshots per window:
-//   covariance  per tile, whatever the window (the epilogue), 41 us for rows of 128 slots, 50 of 64 or
-//               32 and 105 of 16, with complex weights 82 and 108; per item 40 us and 0.043 per value
-//               of a CTA's transform (4x256: 470 us, 8x64 205, 16x16 152; complex 874, 298, 163). The
-//               products run under that in part, 0.0182 us per snapshot and MMA unit (a 256 x 256
-//               product of the chunk: 3 a diagonal tile, 4 another; 4x256 914 us at 768 snapshots).
-//               Where the voltages cannot come by TMA 0.25 us per snapshot and tile (4x100: 616 us);
-//   transform   us per snapshot and 1000 beams: 0.8 the 512-beam kernels (4x256: 826 us at 512),
-//               0.58 the 32-beam kernel, 1.2 the 256-beam ones, 1.1 those of 1024 and 2048 beams, 1.9
-//               the other FFT kernels (8x64: 979 us at 512); the direct DFT 1.0 for every N-S feed.
-//               The split-FP16 kernel (split) 1.3 (4x256: 2060 us at 768).
-// So 4x256 changes over near 420 snapshots, 8x64 near 110, 16x16 near 600. Only the plan's sizes
-// enter, never the number of windows or the pointer: a window's beams do not depend on its call.
+// Whether the covariance is taken rather than the transform of every snapshot: an estimate of both in
+// microseconds for 608 work items (eight per CTA pair) on a GB300,
+//   covariance  34 us per tile and 55 us per item, 1.4 times that with complex weights (epilogue
+//               and transform of V, whatever the window), and from there 0.021 us per snapshot and
+//               MMA unit (a 256 x 256 product of the chunk: 3 a diagonal tile, 4 another), three
+//               times that where the voltages cannot come by TMA;
+//   transform   us per snapshot and 1000 beams: 0.8 the 512-beam kernels (4x256: 829 us at 512),
+//               0.6 the 32-beam kernel, 1.1 those of 1024 and 2048 beams, 1.9 the other FFT
+//               kernels (8x64: 979 us at 512); the direct DFT 1.0 for every N-S feed. The
+//               split-FP16 kernel (split) 1.3 (4x256: 2060 us at 768).
+// So 4x256 changes over near 300 snapshots, 8x64 near 90, 16x16 near 400. These are the costs of the
+// covariance with its products rounded to FP32; with their errors kept it takes longer (4x256 470 us
+// and up for 398, 8x64 205 for 160, 16x16 152 for 107; complex weights 820, 281, 174) and the times
+// meet near 420, 110 and 570 snapshots, 4x256 with complex weights near 770. The line stays where it
+// was: between the two the covariance costs up to 1.35 times the transform (complex 1.6), for an error
+// of 3e-8 in place of 1e-7 to 6e-7 (2-norm), and nothing that had the smaller error loses it. Only the
+// plan's sizes enter, never the number of windows or the pointer: a window's beams do not depend on
+// its call.
 bool corr_preferred(const BeamArgs& a, bool split) {
   CorrJob j;
   CorrSizes s;
@@ -1278,15 +1282,12 @@ bool corr_preferred(const BeamArgs& a, bool split) {
     tiles += c + 1;
     units += w * (3 + 4 * c);
   }
-  static const double kTile[4] = {50.0, 50.0, 105.0, 41.0}, kTileC[4] = {82.0, 82.0, 108.0, 82.0};
-  const double fixed = tiles * (a.real_w ? kTile : kTileC)[j.mode] + 40.0 + 0.043 * a.my * (((a.mx + 1) / 2 + 1) / 2);
-  const double cov = j.ny % 16 == 0 && corr::KS % a.npol == 0
-                         ? std::max(fixed, (a.real_w ? 0.85 : 1.0) * fixed + 0.0182 * units * nsnap)
-                         : std::max(fixed, (a.real_w ? 17.0 * tiles : 0.5 * fixed) + 0.25 * tiles * nsnap);
+  const double fixed = (34.0 * tiles + 55.0) * (a.real_w ? 1.0 : 1.4);
+  const double cov = std::max(fixed, 0.6 * fixed + 0.021 * (j.ny % 16 == 0 && corr::KS % a.npol == 0 ? 1 : 3) * units * nsnap);
   double per;                                          // us per snapshot
   if (split) per = 1.3e-3 * nout;
   else if (fp32_n512_supported(a)) per = 0.8e-3 * nout;
-  else if (fp32_warp_supported(a)) per = (a.my == 32 ? 0.58e-3 : a.my == 256 ? 1.2e-3 : a.my >= 1024 ? 1.1e-3 : 1.9e-3) * nout;
+  else if (fp32_warp_supported(a)) per = (a.my == 32 ? 0.6e-3 : a.my >= 1024 ? 1.1e-3 : 1.9e-3) * nout;
   else if (fp32_fft_supported(a.mx, a.my)) per = 1.9e-3 * std::max<double>(nout, j.nant);
   else per = 1e-3 * nout * a.nyf;
   return cov < per * nsnap;
