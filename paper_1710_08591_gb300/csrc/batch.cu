@@ -13,7 +13,7 @@
 // a CUDA graph and replayed while the batch's buffers stay the same.
 // Arrays with windows of many snapshots (corr_preferred) go through the covariance kernel
 // instead, all of them in one launch over a job table of its own, in the same graph: twelve
-// uneven arrays of 512 snapshots per window 20.99 -> 11.63 ms (all twelve through it).
+// uneven arrays of 512 snapshots per window 20.99 -> 12.86 ms (all twelve through it).
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -44,9 +44,9 @@
 // about 128 bytes per cycle), and between tiles the epilogue, about 4500 cycles per half with real
 // weights: a third its products, a third the gather of the lags. Measured on a GB300 (the FFT
 // kernels; this one with products and sums rounded to FP32; this one): 4x256, 2 polarisations,
-// 4096 windows x channels of 768 snapshots 8.57, 5.20, 6.09 ms (the MMAs alone would need 3.3 ms, 540
+// 4096 windows x channels of 768 snapshots 8.57, 5.20, 6.16 ms (the MMAs alone would need 3.3 ms, 540
 // tiles of 6.1 us in turn); 16 such items 608, 104, 119 us; 8x64 with complex gains, 2048 items of 512
-// snapshots 3.44, 0.90, 1.17 ms; 3x37 onto 5x73 beams, 360 items of 100 snapshots 1267, 143, 139 us.
+// snapshots 3.44, 0.90, 1.19 ms; 3x37 onto 5x73 beams, 360 items of 100 snapshots 1267, 143, 139 us.
 // Largest error of a beam beside a source of amplitude 7 over noise of 0.3, 4x256 with half-sine
 // weights: 2e-6, 1e-4, 6e-8.
 // An item's sums are whole numbers or taken in an order that depends on the item alone, so its
