@@ -1151,8 +1151,8 @@ bool corr_make_job(const BeamArgs& a, CorrJob* J) {
   // is 2^-19 of that, and with n = nx ny ceil(nx / mx) feed pairs of one separation above 1024 2^e
   // times it (n <= 1024 2^e): V stays below 2^30 units. What lies below a unit, at most 1/2 + 2^-5 a
   // product and 1.4 with complex weights, sums over up to 2 n of them to 1.4 2^(11 + e) units at most,
-  // and is kept in 2^-(19 - e) of one: below 2^31. With e = 4 that is 2^-30 of the largest product, rounded once for
-  // every 16 or more of them; lattices folded further take the transform.
+  // and is kept in 2^-(19 - e) of one: below 2^31. With e = 4 that is 2^-30 of the largest product,
+  // rounded once for every 16 or more of them; lattices folded further take the transform.
   auto clog2 = [](int64_t n) { int l = 0; while (((int64_t)1 << l) < n) ++l; return l; };
   const int ns = clog2(nsnap), e = std::max(0, clog2((int64_t)j.nant * ((a.nx + a.mx - 1) / a.mx)) - 10);
   const int z = a.real_w ? 0 : 31 - ns, w = a.w_exp == kNoExp ? 0 : a.w_exp;
